@@ -98,7 +98,7 @@ struct rkm_ctx {
     // bucket sort scratch
     Buf hist, offs;
     // threshold pass
-    Buf cand, cand_cnt, lfin, keys, kid, topk_tmp;
+    Buf cand, cand_cnt, lfin, topk_tmp;
     // threshold pass: seed bounds and user order
     Buf lseed, thr_perm;
     // counting pass
@@ -110,7 +110,7 @@ struct rkm_ctx {
     int64_t res_n = 0;
     int res_d = 0;
     unsigned res_off_grid = 0;
-    Buf res_U, res_e, res_q, res_tau, res_tid, res_uperm, res_ucum, res_pack, res_meta;
+    Buf res_U, res_e, res_q, res_nrm, res_tau, res_tid, res_uperm, res_ucum, res_pack, res_meta;
     // query scratch
     Buf q_e, q_q, q_n2, q_nrm, q_nhat, q_del, q_perm, q_pack, q_tmax, q_thmax, q_tdel, q_cnt, q_texp;
     // host staging for rkm_topn_host
@@ -214,9 +214,9 @@ struct rkm_ctx {
     void free_all() {
         Buf* all[] = {&topk_tmp, &u_e, &u_q, &u_n2, &u_nrm, &u_nhat, &u_del, &u_pack, &p_e, &p_q, &p_n2, &p_nrm,
                       &p_nhat, &p_del, &p_perm, &p_pack, &tmax, &thmax, &tdel, &hist, &offs, &cand,
-                      &cand_cnt, &lfin, &keys, &kid, &r_u, &uperm, &ucum, &us_pack, &us_meta,
+                      &cand_cnt, &lfin, &r_u, &uperm, &ucum, &us_pack, &us_meta,
                       &nprefix, &unit_off, &band, &cnt_s, &top_ids, &top_sc, &lseed, &thr_perm,
-                      &tau_tmp, &tid_tmp, &res_U, &res_e, &res_q, &res_tau, &res_tid, &res_uperm, &res_ucum,
+                      &tau_tmp, &tid_tmp, &res_U, &res_e, &res_q, &res_nrm, &res_tau, &res_tid, &res_uperm, &res_ucum,
                       &res_pack, &res_meta, &q_e, &q_q,
                       &q_n2, &q_nrm, &q_nhat, &q_del, &q_perm, &q_pack, &q_tmax, &q_thmax, &q_tdel, &q_cnt,
                       &q_texp, &p_texp,
@@ -538,8 +538,6 @@ struct ThrPlan {
     Cand* cand;
     int* cand_cnt;
     unsigned* lfin;
-    unsigned long long* keys;
-    int* kid;
     int nseg, cap;
 };
 
@@ -563,8 +561,6 @@ rkm_status threshold_prepare(rkm_ctx* c, const PathShape& ps, const float* U, in
     TRY(c->ensure(c->cand, n * (int64_t)pl->nseg * pl->cap, &pl->cand));
     TRY(c->ensure(c->cand_cnt, n * (int64_t)pl->nseg, &pl->cand_cnt));
     TRY(c->ensure(c->lfin, n, &pl->lfin));
-    TRY(c->ensure(c->keys, n * (int64_t)pl->nseg * pl->cap, &pl->keys));
-    TRY(c->ensure(c->kid, n * (int64_t)pl->nseg * pl->cap, &pl->kid));
     CUDA_TRY(cudaMemsetAsync(pl->lfin, 0, n * sizeof(unsigned), s));
     CUDA_TRY(cudaMemsetAsync(pl->cand_cnt, 0, n * pl->nseg * sizeof(int), s));
     ThresholdArgs& a = pl->a;
@@ -629,9 +625,9 @@ void threshold_exact(rkm_ctx* c, const float* U, int64_t ldu, const float* P, in
                      cudaStream_t s) {
     Phase ph(c, s, RKM_PHASE_EXACT);
     ExactData x{U, ldu, up.e, up.q, P, ldp, it.rp.e, it.rp.q, d, (int)round_up(d, 8), &c->st->off_grid,
-                pl.a.n, it.m};
-    launch_exact_tau(x, pl.cand, pl.cand_cnt, pl.lfin, pl.cap, pl.nseg, it.perm, pl.a.n, pl.a.k, pl.keys, pl.kid,
-                     tau, tid, topk, c->st, s, pl.a.uperm);
+                pl.a.n, it.m, up.nrm, it.tmax};
+    launch_exact_tau(x, pl.cand, pl.cand_cnt, pl.lfin, pl.cap, pl.nseg, it.perm, pl.a.n, pl.a.k, tau, tid, topk,
+                     c->st, s, pl.a.uperm);
 }
 
 // Seed order of the tensor-core threshold pass.  Items arrive in descending norm order and a
@@ -687,8 +683,8 @@ rkm_status grow_candidates(rkm_ctx* c, int64_t m, int attempt) {
     return RKM_OK;
 }
 
-// Device bytes the candidate lists of one threshold launch may take (20 bytes per slot:
-// the candidate, its exact key and its id): half of the device memory, at most 48 GB.
+// Device bytes the candidate lists of one threshold launch may take (one Cand per slot): half
+// of the device memory, at most 48 GB.
 int64_t candidate_budget(const rkm_ctx* c) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -711,7 +707,7 @@ rkm_status thresholds_core(rkm_ctx* c, const PathShape& ps, const float* U, int6
                            const float* P, int64_t ldp, int d, int k, const RowPrep& up, const ItemSide& it,
                            double* tau, int* tid, int* topk, cudaStream_t s) {
     for (int attempt = 0;; ++attempt) {
-        const int64_t per_user = (int64_t)threshold_segments(ps, k, c->opts.epilogue_groups) * c->cand_cap * 20;
+        const int64_t per_user = (int64_t)threshold_segments(ps, k, c->opts.epilogue_groups) * c->cand_cap * (int64_t)sizeof(Cand);
         const int64_t slice = std::min<int64_t>(n, std::max<int64_t>(BU, candidate_budget(c) / per_user / BU * BU));
         bool overflow = false;
         for (int64_t u0 = 0; u0 < n && !overflow; u0 += slice) {
@@ -923,7 +919,7 @@ rkm_status rkm::query_resident(rkm_ctx* c, const rkm_ctx* r, const float* Q, int
                  static_cast<UserMeta*>(r->res_meta.p)};
     ExactData x{static_cast<const float*>(r->res_U.p), d, static_cast<const int*>(r->res_e.p),
                 static_cast<const int16_t*>(r->res_q.p), Q, ldq, it.rp.e, it.rp.q, d, (int)round_up(d, 8),
-                &c->st->off_grid, n, q};
+                &c->st->off_grid, n, q, static_cast<const float*>(r->res_nrm.p), it.tmax};
     int* cnt;
     TRY(c->ensure(c->q_cnt, q, &cnt));
     for (int attempt = 0;; ++attempt) {
@@ -1078,7 +1074,7 @@ rkm_status count_prepare(rkm_ctx* c, const PathShape& ps, const float* U, int64_
                         &cp->uo, s));
     }
     cp->x = ExactData{U, ldu, up.e, up.q, P, ldp, it.rp.e, it.rp.q, d, (int)round_up(d, 8), &c->st->off_grid,
-                      n, it.m};
+                      n, it.m, up.nrm, it.tmax};
     TRY(c->ensure(c->cnt_s, it.m, &cp->cnt));
     return RKM_OK;
 }
@@ -1449,7 +1445,7 @@ rkm_status rkm_resident_set(rkm_ctx* c, const float* U, int64_t n, int64_t ldu, 
         CUDA_TRY(cudaMemcpyAsync(tid_c, tid, n * sizeof(int), cudaMemcpyDeviceToDevice, s));
     }
     RowPrep up;
-    TRY(prep_rows(c, ps, Uc, n, d, d, c->res_e, c->res_q, c->u_n2, c->u_nrm, c->u_nhat, c->u_del, &up, s));
+    TRY(prep_rows(c, ps, Uc, n, d, d, c->res_e, c->res_q, c->u_n2, c->res_nrm, c->u_nhat, c->u_del, &up, s));
     UserOrder uo;
     TRY(order_users(c, ps, Uc, n, d, d, up, tau_c, tid_c,
                     UserBufs{c->res_uperm, c->res_ucum, c->res_pack, c->res_meta},
@@ -1613,7 +1609,7 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
         BatchJob& j = J[i];
         j = BatchJob{};
         j.x = ExactData{I.U, I.ldu, x.up.e, x.up.q, I.P, I.ldp, x.it.rp.e, x.it.rp.q, I.d, (int)round_up(I.d, 8),
-                        &sc->st->off_grid, I.n, I.m};
+                        &sc->st->off_grid, I.n, I.m, x.up.nrm, x.it.tmax};
         j.cand = x.pl.cand;
         j.cand_cnt = x.pl.cand_cnt;
         j.lfin = x.pl.lfin;
@@ -1624,8 +1620,6 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
         j.m = I.m;
         j.k = I.k;
         j.N = I.N;
-        j.keys = x.pl.keys;
-        j.kid = x.pl.kid;
         j.tau = x.tau;
         j.tid = x.tid;
         j.user_begin = users;

@@ -173,14 +173,16 @@ struct ExactData {
     const unsigned* off_grid;  // device flag: zero = every row on the grid, use the integer path
     // Debug builds check gathered indices against these (0 = unchecked).
     int64_t n_users = 0, m_items = 0;
+    const float* unrm = nullptr;  // [n] ||u|| rounded up, original order
+    const float* pmax = nullptr;  // largest ||p|| of the first item tile (rounded up)
 };
 
 // K3: exact tau_u, t_u and (optionally) S_k(u) from the candidate lists.  With uperm, the
 // lists are by threshold-pass row and uperm[row] is the original user (rows, outputs).
 void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt, const unsigned* lfin_key,
                       int cap, int nseg, const int* item_perm, int64_t n, int k,
-                      unsigned long long* keys, int* kid, double* tau, int* tid, int* topk,
-                      DevStatus* st, cudaStream_t s, const int* uperm = nullptr);
+                      double* tau, int* tid, int* topk, DevStatus* st, cudaStream_t s,
+                      const int* uperm = nullptr);
 
 // K6: rescore queued band pairs (orig user, sorted item pos) and add members to counts.
 void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap,
@@ -257,8 +259,6 @@ struct BatchJob {
     const int* item_perm;         // sorted pos -> item id
     int64_t n, m;
     int k, N;
-    unsigned long long* keys;
-    int* kid;
     double* tau;
     int* tid;
     int64_t user_begin;           // first user of this problem in the launch's numbering
