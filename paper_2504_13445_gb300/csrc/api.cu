@@ -601,10 +601,11 @@ rkm_status threshold_descriptor(const PathShape& ps, const ThrPlan& pl, const It
     return RKM_OK;
 }
 
-// slot: descriptor slot (0 or 1; the seed pass and the main pass of one call use different
-// slots, since the pinned staging of the first may not have been copied yet).
+// The seed pass and the main pass of one call use different descriptor slots, since the pinned
+// staging of the first may not have been copied yet.
 rkm_status threshold_launch_one(rkm_ctx* c, const PathShape& ps, const ThrPlan& pl, const ItemSide& it,
-                                cudaStream_t s, int slot = 0) {
+                                cudaStream_t s, bool seed = false) {
+    const int slot = seed ? 1 : 0;
     Phase ph(c, s, RKM_PHASE_THRESHOLD);
     c->stats.threshold_launches++;
     if (ps.tc) {
@@ -613,7 +614,7 @@ rkm_status threshold_launch_one(rkm_ctx* c, const PathShape& ps, const ThrPlan& 
         TRY(c->instances(2, &hi, &di));
         TRY(threshold_descriptor(ps, pl, it, hi + slot));
         CUDA_TRY(cudaMemcpyAsync(di + slot, hi + slot, sizeof(TcInstance), cudaMemcpyHostToDevice, s));
-        launch_threshold_tc(di + slot, 1, (pl.a.n + BU - 1) / BU, pl.a.k, ps.dp, ps.fp8, pl.nseg, c->num_sms, s);
+        launch_threshold_tc(di + slot, 1, (pl.a.n + BU - 1) / BU, pl.a.k, ps.dp, ps.fp8, pl.nseg, seed, c->num_sms, s);
     } else {
         launch_threshold_simt(pl.a, s);
     }
@@ -632,22 +633,31 @@ void threshold_exact(rkm_ctx* c, const float* U, int64_t ldu, const float* P, in
 
 // Seed order of the tensor-core threshold pass.  Items arrive in descending norm order and a
 // user tile stops once no user of it can still reach its bound (Algorithm 1's Cauchy-Schwarz
-// stop), so a tile stops as late as its user with the smallest tau_u / ||u||.  A first pass
-// of the same kernel over the SEED_TILES highest-norm item tiles gives every user a lower
-// bound L_u of tau_u (the k-th largest lower bound over those items); users are then packed
-// in the order of L_u / ||u||, so that the users of a tile stop at about the same item, and
-// L_u seeds the selector of the main pass.  The results do not depend on the order.  Used when
-// a tile's product is two K-blocks deep or more (BF16 d > 64): measured on GB300 at
-// 2M x 500K, d = 128, the products computed fell from 59 % to 52 % of n*m and the threshold
-// phase from 116 to 104 ms; at 500K x 100K, d = 64, where the epilogue bounds the kernel, the
-// phase grew from 7.9 to 8.9 ms.
-#ifndef RKM_SEED_TILES
-#define RKM_SEED_TILES 8
-#endif
-constexpr int64_t SEED_TILES = RKM_SEED_TILES;
+// stop), so a tile stops as late as its user with the smallest tau_u / ||u||.  A first pass over
+// the highest-norm item tiles gives every user a lower bound L_u of tau_u; users are then packed
+// in the order of L_u / ||u||, so that the users of a tile stop at about the same item, and L_u
+// seeds the selector of the main pass, which then records few of the candidates that a bound
+// growing from nothing lets through.  The results do not depend on the order.
+//
+// Tiles of the seed pass (0 = none): 16 / 8 / 4 with one / two / more K-blocks per tile, twice as
+// many for k >= 32, at most 16 and a sixth of the items; none unless they give 2 k values (16 per
+// tile) to take the k-th of.  Threshold phase on GB300 (ms) with 4 / 8 / 16 / 32 seed tiles:
+//   500K x 100K, d = 64,  k = 25   5.84  5.01  4.81  4.94   (6.48 without)
+//   2M x 500K,   d = 128, k = 10   83.8  79.1  79.2  81.1   (91.3 with a recording seed pass)
+//   200K x 50K,  d = 96,  k = 20   2.11  1.96  1.98  2.12   (2.84)
+//   130K x 30K,  d = 100, k = 50   1.96  1.74  1.61  1.68   (2.97)
+//   480K x 18K,  d = 200, k = 10   3.67  3.81  4.16  4.89   (4.57)
+//   100K x 50K,  d = 128, FP8      3.11  2.59  2.38  2.37   (3.74)
+int64_t seed_tiles(const PathShape& ps, int64_t item_tiles, int k) {
+    const int64_t kblocks = ps.dp * ps.elem_bytes / 128;
+    int64_t t = std::max<int64_t>(4, 16 / kblocks);
+    if (k >= 32) t *= 2;
+    t = std::min<int64_t>(std::min<int64_t>(t, 16), item_tiles / 6) & ~(int64_t)1;
+    return 16 * std::min<int64_t>(t, 8) >= 2 * k ? t : 0;
+}
 
 rkm_status threshold_seed_order(rkm_ctx* c, const PathShape& ps, const float* U, int64_t n, int64_t ldu, int d,
-                                const RowPrep& up, const ItemSide& it, ThrPlan* pl, cudaStream_t s) {
+                                const RowPrep& up, const ItemSide& it, ThrPlan* pl, int64_t tiles, cudaStream_t s) {
     unsigned *seed, *hist, *offs;
     float* r;
     int* perm;
@@ -656,11 +666,10 @@ rkm_status threshold_seed_order(rkm_ctx* c, const PathShape& ps, const float* U,
     TRY(c->ensure(c->hist, HIST_WORDS, &hist));
     TRY(c->ensure(c->offs, NBUCKET, &offs));
     TRY(c->ensure(c->thr_perm, n, &perm));
-    CUDA_TRY(cudaMemsetAsync(seed, 0, n * sizeof(unsigned), s));
     ThrPlan pre = *pl;
-    pre.a.m = std::min<int64_t>(it.m, SEED_TILES * BI_TC);
+    pre.a.m = tiles * BI_TC;
     pre.a.lfin_key = seed;
-    TRY(threshold_launch_one(c, ps, pre, it, s, 1));
+    TRY(threshold_launch_one(c, ps, pre, it, s, true));
     {
         Phase ph(c, s, RKM_PHASE_PREP);
         launch_seed_ratio(seed, up.nrm, n, r, s);
@@ -715,9 +724,8 @@ rkm_status thresholds_core(rkm_ctx* c, const PathShape& ps, const float* U, int6
             const RowPrep us = row_slice(up, u0, d);
             ThrPlan pl;
             TRY(threshold_prepare(c, ps, U + u0 * ldu, un, ldu, d, k, us, it, &pl, s));
-            if (ps.tc && c->opts.seed_order && slice >= n && it.tiles >= 2 * SEED_TILES &&
-                ps.dp * ps.elem_bytes >= 256)
-                TRY(threshold_seed_order(c, ps, U, n, ldu, d, up, it, &pl, s));
+            const int64_t seeds = ps.tc && c->opts.seed_order && slice >= n ? seed_tiles(ps, it.tiles, k) : 0;
+            if (seeds > 0) TRY(threshold_seed_order(c, ps, U, n, ldu, d, up, it, &pl, seeds, s));
             TRY(threshold_launch_one(c, ps, pl, it, s));
             threshold_exact(c, U + u0 * ldu, ldu, P, ldp, d, us, it, pl, tau + u0, tid + u0,
                             topk ? topk + u0 * k : nullptr, s);
@@ -1754,7 +1762,7 @@ rkm_status batch_enqueue(rkm_ctx* c, const rkm_instance* inst, int count, cudaSt
             units += (inst[i].n + BU - 1) / BU;
         }
         CUDA_TRY(cudaMemcpyAsync(dev, c->batch_host, (size_t)count * sizeof(TcInstance), cudaMemcpyHostToDevice, s));
-        launch_threshold_tc(dev, count, units, kheap, max_dp, w[0].ps.fp8, nseg, c->num_sms, s);
+        launch_threshold_tc(dev, count, units, kheap, max_dp, w[0].ps.fp8, nseg, false, c->num_sms, s);
         return batch_enqueue_tc(c, inst, count, w, max_dp, s);
     } else {
         for (int i = 0; i < count; ++i) launch_threshold_simt(w[i].pl.a, s);

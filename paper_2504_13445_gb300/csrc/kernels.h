@@ -135,8 +135,10 @@ int threshold_groups(int kheap, int max_dp, bool fp8, int want);
 // Epilogue warpgroups of the tensor-core counting kernel for padded depth dp (want as above).
 int count_groups(int dp, bool fp8, int want);
 // ng: epilogue warpgroups, as threshold_groups returned for these instances.
+// seed: the pass that only bounds tau_u from below over a.m items (an even number of whole tiles,
+// k <= 64) and writes float_key of the bound to a.lfin_key[user]; it records no candidates.
 void launch_threshold_tc(const TcInstance* inst, int count, long long total_units, int kheap, int max_dp,
-                         bool fp8, int ng, int num_sms, cudaStream_t s);
+                         bool fp8, int ng, bool seed, int num_sms, cudaStream_t s);
 
 // Approximate products of the tensor-core paths with their guard band, for validating the
 // error bound: v[u * ldo + perm[pos]] = the product the threshold and counting kernels see

@@ -46,6 +46,7 @@ struct TcBars {
     uint64_t res_full[2], res_empty[2], drain;
     uint64_t full[MAX_SLOTS], empty[MAX_SLOTS];
     uint64_t tfull[2], tempty[2];
+    uint64_t xfull, xempty;  // seed pass: exchange of the warpgroups' values
     uint32_t tmem_base;
     int abort;
     // Threshold pass, early end of a unit (see k_threshold_tc): the producer's end marker in
@@ -149,6 +150,8 @@ __device__ __forceinline__ void setup(TcBars* B, int slots, int warp, int consum
             mbar_init(&B->tfull[b], 1);
             mbar_init(&B->tempty[b], (uint32_t)consumers);
         }
+        mbar_init(&B->xfull, 4);
+        mbar_init(&B->xempty, 4);
         B->abort = 0;
         mbar_fence_init();
     }
@@ -184,11 +187,42 @@ __device__ __forceinline__ int unit_instance(const TcInstance* inst, int count, 
     return lo;
 }
 
+// Seed pass: values per row and warpgroup, and its shared exchange buffer [SEED_SLOTS][BU].
+constexpr int SEED_SLOTS = 64;
+
+// v sorted in descending order (bitonic network over registers); from: first merge size.
+template <int FROM>
+__device__ __forceinline__ void sort64_desc(float (&v)[SEED_SLOTS]) {
+#pragma unroll
+    for (int size = FROM; size <= SEED_SLOTS; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll
+            for (int i = 0; i < SEED_SLOTS; ++i) {
+                const int j = i ^ stride;
+                if (j > i) {
+                    const float hi = fmaxf(v[i], v[j]), lo = fminf(v[i], v[j]);
+                    const bool desc = (i & size) == 0;
+                    v[i] = desc ? hi : lo;
+                    v[j] = desc ? lo : hi;
+                }
+            }
+        }
+    }
+}
+
 // Threshold pass over one or many independent problems.  Work units are (instance, user
 // tile) pairs numbered consecutively across the instances; CTA b takes units b, b + grid, ...
 // A unit streams every item tile of its instance, so the caller orders the instances by
 // descending cost to balance the CTAs.
-template <bool FP8, int NG>
+// SEED: the lower bounds of tau_u that start the pass, from the leading item tiles alone (a.m
+// is an even number of whole tiles).  Nothing is recorded: every 16 columns give one value, the
+// maximum that the TMEM load returns less the tile's error bound; the two warpgroups keep 64 of
+// them each per row (a value per 16, 32, ... items as tiles are added), and the k-th largest of
+// the 128 bounds tau_u, because k distinct items reach it.  A seed pass that recorded candidates and
+// kept heaps took 24,000 to 97,000 cycles per tile and warpgroup on its first tiles (6 % of the
+// threshold phase at 2M x 500K, 45 % at 130K x 30K, k = 50); this one 1,000 to 2,500.
+template <bool FP8, int NG, bool SEED>
 __global__ void __launch_bounds__(tc_threads(NG), 1)
     k_threshold_tc(const TcInstance* __restrict__ inst, int count, long long total_units, int kheap,
                    const TcLayout L) {
@@ -206,7 +240,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
     // the work unit (a bound of another unit is never used).  Initialised before setup's
     // barrier so that no group can read an uninitialised entry.
     unsigned long long* Lpub = reinterpret_cast<unsigned long long*>(heaps + NG * kheap * BU);
-    if (warp >= 2) Lpub[threadIdx.x - 64] = 0xFFFFFFFF00000000ull;
+    if (!SEED && warp >= 2) Lpub[threadIdx.x - 64] = 0xFFFFFFFF00000000ull;
     if (threadIdx.x < 16) {
         B->need_pub[threadIdx.x] = 0xFFFFFFFF00000000ull;
         B->tmark[threadIdx.x] = 0;
@@ -242,7 +276,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                     // Stop the unit when no user of it needs the remaining tiles (at least two
                     // remaining, so that both end markers fall inside the unit's tile range):
                     // the first ring slot of tile `it` then carries an end marker, no copy.
-                    if (it + 1 < item_tiles && it >= unit_stop(B, (unsigned)w, item_tiles, NG)) {
+                    if (!SEED && it + 1 < item_tiles && it >= unit_stop(B, (unsigned)w, item_tiles, NG)) {
                         if (!mbar_wait(&B->empty[slot], ph ^ 1u, abort, st)) {
                             ok = false;
                             break;
@@ -359,6 +393,80 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             tc_commit(&B->drain);
             drain_wait(&B->drain, 0u, st);
         }
+    } else if constexpr (SEED) {
+        static_assert(!SEED || NG == 2, "the seed pass runs two warpgroups");
+        const int h = (warp - 2) >> 2;  // warpgroup = accumulator buffer
+        const int q = warp & 3;
+        const int r = q * 32 + lane;
+        uint32_t use = 0, xphase = 0;
+        bool ok = true;
+        for (long long w = blockIdx.x; w < total_units && ok; w += gridDim.x, xphase ^= 1u) {
+            const TcInstance& I = inst[unit_instance(inst, count, w)];
+            const ThresholdArgs& a = I.a;
+            const int64_t u = (w - I.unit_begin) * BU + r;
+            const bool active = u < a.n;
+            const float un = active ? a.unrm[u] : 0.f, unh = active ? a.unhat[u] : 0.f;
+            const float ud = active ? a.udel[u] : 0.f;
+            const int ue = (FP8 && active) ? fp8_exp(a.uexp[u]) : 0;
+            const int item_tiles = (int)(a.m / BI_TC);
+            float v[SEED_SLOTS];
+#pragma unroll
+            for (int i = 0; i < SEED_SLOTS; ++i) v[i] = -INFINITY;
+#pragma unroll 1
+            for (int it0 = h; it0 < item_tiles && ok; it0 += 8) {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int it = it0 + 2 * t;
+                    if (it >= item_tiles || !ok) continue;
+                    const float E = err_bound(a.cacc, a.eabs, un, unh, ud, a.thmax[it], a.tdel[it]);
+                    const float f = FP8 ? pow2i(ue + a.texp[it] - 16) : 1.f;
+                    if (!mbar_wait(&B->tfull[h], use & 1u, abort, a.st)) {
+                        ok = false;
+                        continue;
+                    }
+                    __syncwarp();
+                    tc_fence_after();
+                    const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)h * BI_TC;
+#pragma unroll
+                    for (int c = 0; c < 16; c += 2) {
+                        uint32_t ra[16], rb[16];
+                        float ma, mb;
+                        tmem_ld16_max_issue(tb + c * 16, ra, ma);
+                        tmem_ld16_max_issue(tb + c * 16 + 16, rb, mb);
+                        tmem_wait_bind_max(ra, ma);
+                        tmem_wait_bind_max(rb, mb);
+                        v[t * 16 + c] = fmaxf(v[t * 16 + c], __fsub_rd(FP8 ? ma * f : ma, E));
+                        v[t * 16 + c + 1] = fmaxf(v[t * 16 + c + 1], __fsub_rd(FP8 ? mb * f : mb, E));
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&B->tempty[h]);
+                    ++use;
+                }
+            }
+            if (!ok) break;
+            // The 64 largest of both groups' sorted lists are the larger of v[i] and o[63 - i].
+            sort64_desc<2>(v);
+            if (h == 1) {
+                if (!mbar_wait(&B->xempty, xphase ^ 1u, abort, a.st)) break;
+#pragma unroll
+                for (int i = 0; i < SEED_SLOTS; ++i) heaps[i * BU + r] = v[i];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&B->xfull);
+            } else {
+                if (!mbar_wait(&B->xfull, xphase, abort, a.st)) break;
+#pragma unroll
+                for (int i = 0; i < SEED_SLOTS; ++i) v[i] = fmaxf(v[i], heaps[(SEED_SLOTS - 1 - i) * BU + r]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&B->xempty);
+                sort64_desc<SEED_SLOTS>(v);
+                float kth = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < SEED_SLOTS; ++i)
+                    if (i == a.k - 1) kth = v[i];
+                if (active) a.lfin_key[u] = float_key(kth);
+            }
+        }
     } else {
         constexpr int CW = 2 * BI_TC / NG;  // accumulator columns a group reads per tile
         const int ew = warp - 2;          // 0 .. 4 NG - 1
@@ -392,7 +500,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             s.tag = (unsigned)w;
             s.defer = 1;
             s.mark = 0;
-            bool warm = false;  // warm start done for this unit
+            bool warm = a.lfin_seed != nullptr;  // warm start done for this unit (or seeded)
             int fb = item_tiles;       // first tile after the last searched one whose
             float bnd_fb = -INFINITY;  // ||u|| max||p|| is below bnd_fb (see the stop below)
             // Packed row u holds original user uo; a seed bound of tau_u (from a pass over the
@@ -464,7 +572,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                         if constexpr (FP8) scale_values(v, f);
                     };
                     const float lw = warm_bound<CW / 4, CW>(load, it * BI_TC + cg, a.m, a.k, E);
-                    s.Lw = active ? fmaxf(lw, seed) : -INFINITY;
+                    s.Lw = active ? lw : -INFINITY;
                     publish_bound(s.pub, s.tag, s.Lw);
                     warm = true;
                 }
@@ -1081,17 +1189,18 @@ rkm_status make_tmaps(const void* A, int64_t a_rows, const void* B, int64_t b_ro
 
 namespace {
 
-TcLayout threshold_layout(int ng, int kheap, int max_dp, bool fp8) {
+TcLayout threshold_layout(int ng, int kheap, int max_dp, bool fp8, bool seed) {
     const int KB = fp8 ? max_dp / 128 : max_dp / 64;
+    if (seed) return make_layout(KB * KB_BYTES_U, KB_BYTES_I, SEED_SLOTS * BU * 4u, MAX_SLOTS);
     return make_layout(KB * KB_BYTES_U, KB_BYTES_I, (uint32_t)ng * BU * kheap * 4u + (uint32_t)ng * BU * 8u,
                        MAX_SLOTS);
 }
 
-template <bool FP8, int NG>
+template <bool FP8, int NG, bool SEED>
 void launch_threshold_ng(const TcInstance* inst, int count, long long total_units, int kheap, const TcLayout& L,
                          int grid, cudaStream_t s) {
-    cudaFuncSetAttribute(k_threshold_tc<FP8, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
-    k_threshold_tc<FP8, NG><<<grid, tc_threads(NG), L.bytes, s>>>(inst, count, total_units, kheap, L);
+    cudaFuncSetAttribute(k_threshold_tc<FP8, NG, SEED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
+    k_threshold_tc<FP8, NG, SEED><<<grid, tc_threads(NG), L.bytes, s>>>(inst, count, total_units, kheap, L);
 }
 
 }  // namespace
@@ -1102,7 +1211,7 @@ void launch_threshold_ng(const TcInstance* inst, int count, long long total_unit
 // longer), and 18 warps leave 96 registers per thread, so the hit path spills.
 int threshold_groups(int kheap, int max_dp, bool fp8, int want) {
     if (want != 4 || kheap > 32) return 2;
-    return threshold_layout(4, kheap, max_dp, fp8).slots >= 2 ? 4 : 2;
+    return threshold_layout(4, kheap, max_dp, fp8, false).slots >= 2 ? 4 : 2;
 }
 
 // Four groups for BF16 tiles one K-block deep (d <= 64): the MMA of a tile is then shortest and
@@ -1115,18 +1224,21 @@ int count_groups(int dp, bool fp8, int want) {
 }
 
 void launch_threshold_tc(const TcInstance* inst, int count, long long total_units, int kheap, int max_dp,
-                         bool fp8, int ng, int num_sms, cudaStream_t s) {
-    if (ng != 4) ng = 2;
-    const TcLayout L = threshold_layout(ng, kheap, max_dp, fp8);
+                         bool fp8, int ng, bool seed, int num_sms, cudaStream_t s) {
+    if (ng != 4 || seed) ng = 2;
+    const TcLayout L = threshold_layout(ng, kheap, max_dp, fp8, seed);
     const int grid = (int)(total_units < num_sms ? total_units : num_sms);
     if (grid < 1) return;
     note_launch();
-    if (fp8) {
-        if (ng == 4) launch_threshold_ng<true, 4>(inst, count, total_units, kheap, L, grid, s);
-        else launch_threshold_ng<true, 2>(inst, count, total_units, kheap, L, grid, s);
+    if (seed) {
+        if (fp8) launch_threshold_ng<true, 2, true>(inst, count, total_units, kheap, L, grid, s);
+        else launch_threshold_ng<false, 2, true>(inst, count, total_units, kheap, L, grid, s);
+    } else if (fp8) {
+        if (ng == 4) launch_threshold_ng<true, 4, false>(inst, count, total_units, kheap, L, grid, s);
+        else launch_threshold_ng<true, 2, false>(inst, count, total_units, kheap, L, grid, s);
     } else {
-        if (ng == 4) launch_threshold_ng<false, 4>(inst, count, total_units, kheap, L, grid, s);
-        else launch_threshold_ng<false, 2>(inst, count, total_units, kheap, L, grid, s);
+        if (ng == 4) launch_threshold_ng<false, 4, false>(inst, count, total_units, kheap, L, grid, s);
+        else launch_threshold_ng<false, 2, false>(inst, count, total_units, kheap, L, grid, s);
     }
 }
 
