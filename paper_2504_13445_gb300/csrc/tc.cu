@@ -9,7 +9,7 @@
 // Roles (64 + 128 NG threads, one CTA per SM, persistent):
 //   warp 0      TMA producer: the resident operand once per work unit, then a ring of
 //               K-block slots of the streamed operand.
-//   warp 1      TMEM allocator and MMA issuer (one thread).
+//   warp 1      TMEM allocator and MMA issuer (one elected lane; see Issuer).
 //   warps 2..   NG epilogue warpgroups.  Group g consumes accumulator buffer g % 2, i.e. every
 //               other product tile, and of each such tile the columns
 //               [(g / 2) * CW, (g / 2 + 1) * CW), CW = 512 / NG.  With NG = 4 every tile is
@@ -174,6 +174,103 @@ __device__ __forceinline__ void teardown(TcBars* B, int warp) {
     }
 }
 
+// State of the MMA issuer (warp 1).  The whole warp runs it on warp-uniform values and one elected
+// lane issues, and the ring slots are unrolled so that barrier addresses and descriptors are
+// constants plus a slot: run by a single lane with a slot index in a register, the barriers,
+// descriptors and commits of a K-block took 750 cycles against its 512 cycles of MMA, so the
+// tensor pipe idled.  Measured in a loop with the same barriers, copies and TMEM reads, cycles per
+// tile of 1 / 2 / 4 K-blocks (512 / 1,024 / 2,048 of MMA): one lane 1,052 / 1,714 / 3,037; this
+// form 746 / 1,068 / 2,127.
+struct Issuer {
+    uint32_t full0, empty0, tfull0, tempty0;  // shared-memory addresses of the barriers
+    uint32_t ringlo, reslo;                   // low descriptor words of the ring and resident buffers
+    uint32_t tmem, idesc;
+    uint32_t slot, ph;                        // next ring slot and the parity of its fill
+    uint32_t b, bph;                          // next accumulator buffer and parity
+    volatile int* abort;
+
+    __device__ __forceinline__ Issuer(TcBars* B, const uint8_t* ring, const uint8_t* res, uint32_t tmem_, uint32_t idesc_)
+        : full0(smem_u32(&B->full[0])), empty0(smem_u32(&B->empty[0])), tfull0(smem_u32(&B->tfull[0])),
+          tempty0(smem_u32(&B->tempty[0])), ringlo(sdesc_lo(smem_u32(ring))), reslo(sdesc_lo(smem_u32(res))),
+          tmem(tmem_), idesc(idesc_), slot(0), ph(0), b(0), bph(1), abort(&B->abort) {}
+
+    // All lanes: the phase completed, or false in all of them when any gave up.
+    __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, DevStatus* st) const {
+        return __all_sync(0xffffffffu, mbar_wait_at(bar, parity, abort, st));
+    }
+
+    __device__ __forceinline__ void turn() {  // the parity turns after buffer 1
+        bph ^= b;
+        b ^= 1u;
+    }
+
+    // The products of one unit: `tiles` tiles of KB K-blocks.  RING_IS_A: the streamed operand is
+    // A (users), else B (items).  MARKS: the producer may end the unit early (see k_threshold_tc).
+    template <bool FP8, int SLOTS, bool RING_IS_A, bool MARKS>
+    __device__ __forceinline__ bool unit(TcBars* B, int tiles, int KB, uint32_t res, int ng, DevStatus* st) {
+        constexpr uint32_t RES = (RING_IS_A ? KB_BYTES_I : KB_BYTES_U) >> 4;
+        constexpr uint32_t RING = (RING_IS_A ? KB_BYTES_U : KB_BYTES_I) >> 4;
+        uint32_t start = slot;
+        int kb = 0;
+        for (;;) {
+#pragma unroll
+            for (uint32_t u = 0; u < (uint32_t)SLOTS; ++u) {
+                if (u < start) continue;
+                if (tiles == 0) {
+                    slot = u;
+                    return true;
+                }
+                bool ok = true;
+                if (kb == 0) ok = mbar_wait_at(tempty0 + b * 8u, bph, abort, st);
+                ok = ok && mbar_wait_at(full0 + u * 8u, ph, abort, st);
+                if (!__all_sync(0xffffffffu, ok)) return false;
+                tc_fence_after();
+                if (MARKS && kb == 0 && *reinterpret_cast<volatile int*>(&B->slot_mark[u]) < 0) {
+                    // The producer ended the unit here: release the marker's slot and pass the end
+                    // to the epilogue warps of both accumulator buffers.
+                    __syncwarp();
+                    if (elect_one()) {
+                        mbar_arrive(&B->empty[u]);
+                        post_unit_end(B, b, 1, ng);
+                    }
+                    turn();
+                    if (!wait(tempty0 + b * 8u, bph, st)) return false;
+                    if (elect_one()) post_unit_end(B, b, 2, ng);
+                    turn();
+                    slot = u + 1u;
+                    if (slot == (uint32_t)SLOTS) {
+                        slot = 0;
+                        ph ^= 1u;
+                    }
+                    return true;
+                }
+                const bool last = kb == KB - 1;
+                if (elect_one()) {
+                    const uint32_t r = ringlo + u * RING, q = res + (uint32_t)kb * RES;
+                    tc_mma_kblock<FP8>(tmem + b * BI_TC, RING_IS_A ? r : q, RING_IS_A ? q : r, idesc, kb == 0);
+                    tc_commit_at(empty0 + u * 8u);
+                    if (last) tc_commit_at(tfull0 + b * 8u);
+                }
+                ++kb;
+                if (last) {
+                    kb = 0;
+                    --tiles;
+                    turn();
+                }
+            }
+            start = 0;
+            ph ^= 1u;
+        }
+    }
+
+    template <bool FP8, bool RING_IS_A, bool MARKS>
+    __device__ __forceinline__ bool unit(TcBars* B, int slots, int tiles, int KB, uint32_t res, int ng, DevStatus* st) {
+        if (slots == 4) return unit<FP8, 4, RING_IS_A, MARKS>(B, tiles, KB, res, ng, st);
+        if (slots == 3) return unit<FP8, 3, RING_IS_A, MARKS>(B, tiles, KB, res, ng, st);
+        return unit<FP8, 2, RING_IS_A, MARKS>(B, tiles, KB, res, ng, st);
+    }
+};
+
 // ---------------------------------------------------------------- K2
 
 // Instance of a work unit w (its global user-tile index): the last instance whose first unit
@@ -319,80 +416,25 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = Op::idesc();
-            int slot = 0;
-            uint32_t ph = 0, tile_j = 0;
-            int iter = 0;
-            bool ok = true;
-            DevStatus* st = inst[0].a.st;
-            for (long long w = blockIdx.x; w < total_units && ok; w += gridDim.x, ++iter) {
-                const TcInstance& I = inst[unit_instance(inst, count, w)];
-                st = I.a.st;
-                const int KB = I.a.dp >> Op::KSHIFT;
-                const int item_tiles = (int)((I.a.m + BI_TC - 1) / BI_TC);
-                const int rb = iter % L.nres;
-                if (!mbar_wait(&B->res_full[rb], (iter / L.nres) & 1, abort, st)) break;
-                tc_fence_after();
-                const uint8_t* sAr = sA + rb * L.res_bytes;
-                for (int it = 0; it < item_tiles && ok; ++it) {
-                    const uint32_t b = tile_j & 1u, use = tile_j >> 1;
-                    if (!mbar_wait(&B->tempty[b], (use & 1u) ^ 1u, abort, st)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    if (!mbar_wait(&B->full[slot], ph, abort, st)) {
-                        ok = false;
-                        break;
-                    }
-                    if (*reinterpret_cast<volatile int*>(&B->slot_mark[slot]) < 0) {
-                        // The producer ended the unit here: release the marker's slot and pass
-                        // the end to the epilogue warps of both accumulator buffers.
-                        mbar_arrive(&B->empty[slot]);
-                        if (++slot == S) {
-                            slot = 0;
-                            ph ^= 1u;
-                        }
-                        post_unit_end(B, b, 1, NG);
-                        ++tile_j;
-                        const uint32_t b2 = tile_j & 1u, use2 = tile_j >> 1;
-                        if (!mbar_wait(&B->tempty[b2], (use2 & 1u) ^ 1u, abort, st)) {
-                            ok = false;
-                            break;
-                        }
-                        post_unit_end(B, b2, 2, NG);
-                        ++tile_j;
-                        break;
-                    }
-                    const uint32_t d = tmem + b * BI_TC;
-                    for (int kb = 0; kb < KB; ++kb) {
-                        if (kb > 0 && !mbar_wait(&B->full[slot], ph, abort, st)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint64_t ad = sdesc_sw128(smem_u32(sAr + kb * KB_BYTES_U));
-                        const uint64_t bd = sdesc_sw128(smem_u32(ring + slot * KB_BYTES_I));
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            Op::mma(d, ad + 2u * k, bd + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
-                        tc_commit(&B->empty[slot]);
-                        if (++slot == S) {
-                            slot = 0;
-                            ph ^= 1u;
-                        }
-                    }
-                    if (!ok) break;
-                    tc_commit(&B->tfull[b]);
-                    ++tile_j;
-                }
-                if (!ok) break;
-                tc_commit(&B->res_empty[rb]);
-            }
+        Issuer q(B, ring, sA, tmem, Op::idesc());
+        int iter = 0;
+        DevStatus* st = inst[0].a.st;
+        for (long long w = blockIdx.x; w < total_units; w += gridDim.x, ++iter) {
+            const TcInstance& I = inst[unit_instance(inst, count, w)];
+            st = I.a.st;
+            const int rb = iter % L.nres;
+            if (!q.wait(smem_u32(&B->res_full[rb]), (iter / L.nres) & 1, st)) break;
+            if (!q.template unit<FP8, false, !SEED>(B, L.slots, (int)((I.a.m + BI_TC - 1) / BI_TC),
+                                                    I.a.dp >> Op::KSHIFT, q.reslo + (uint32_t)rb * (L.res_bytes >> 4), NG,
+                                                    st))
+                break;
+            if (elect_one()) tc_commit(&B->res_empty[rb]);
+        }
+        if (elect_one()) {
             tc_commit(&B->drain);
             drain_wait(&B->drain, 0u, st);
         }
+        __syncwarp();
     } else if constexpr (SEED) {
         static_assert(!SEED || NG == 2, "the seed pass runs two warpgroups");
         const int h = (warp - 2) >> 2;  // warpgroup = accumulator buffer
@@ -832,56 +874,24 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = Op::idesc();
-            int slot = 0;
-            uint32_t ph = 0, tile_j = 0;
-            int iter = 0;
-            bool ok = true;
-            for (long long w = blockIdx.x; w < total && ok; w += gridDim.x, ++iter) {
-                int i, T;
-                int64_t ut0, ut1;
-                cs.decode(w, i, T, ut0, ut1);
-                const int KB = cs.args(i).dp >> Op::KSHIFT;
-                const int rb = iter % L.nres;
-                if (!mbar_wait(&B->res_full[rb], (iter / L.nres) & 1, abort, st0)) break;
-                tc_fence_after();
-                const uint8_t* sBr = sB + rb * L.res_bytes;
-                for (int64_t ut = ut0; ut < ut1 && ok; ++ut) {
-                    const uint32_t b = tile_j & 1u, use = tile_j >> 1;
-                    if (!mbar_wait(&B->tempty[b], (use & 1u) ^ 1u, abort, st0)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t d = tmem + b * BI_TC;
-                    for (int kb = 0; kb < KB; ++kb) {
-                        if (!mbar_wait(&B->full[slot], ph, abort, st0)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint64_t ad = sdesc_sw128(smem_u32(ring + slot * KB_BYTES_U));
-                        const uint64_t bd = sdesc_sw128(smem_u32(sBr + kb * KB_BYTES_I));
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            Op::mma(d, ad + 2u * k, bd + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
-                        tc_commit(&B->empty[slot]);
-                        if (++slot == S) {
-                            slot = 0;
-                            ph ^= 1u;
-                        }
-                    }
-                    if (!ok) break;
-                    tc_commit(&B->tfull[b]);
-                    ++tile_j;
-                }
-                if (!ok) break;
-                tc_commit(&B->res_empty[rb]);
-            }
+        Issuer q(B, ring, sB, tmem, Op::idesc());
+        int iter = 0;
+        for (long long w = blockIdx.x; w < total; w += gridDim.x, ++iter) {
+            int i, T;
+            int64_t ut0, ut1;
+            cs.decode(w, i, T, ut0, ut1);
+            const int rb = iter % L.nres;
+            if (!q.wait(smem_u32(&B->res_full[rb]), (iter / L.nres) & 1, st0)) break;
+            if (!q.template unit<FP8, true, false>(B, S, (int)(ut1 - ut0), cs.args(i).dp >> Op::KSHIFT,
+                                                   q.reslo + (uint32_t)rb * (L.res_bytes >> 4), NG, st0))
+                break;
+            if (elect_one()) tc_commit(&B->res_empty[rb]);
+        }
+        if (elect_one()) {
             tc_commit(&B->drain);
             drain_wait(&B->drain, 0u, st0);
         }
+        __syncwarp();
     } else {
         constexpr int CW = 2 * BI_TC / NG;  // accumulator columns a group reads per tile
         const int ew = warp - 2;
@@ -1123,15 +1133,21 @@ __global__ void k_wait_timeout(long long limit, DevStatus* st) {
     mbar_wait(&bar, 0u, &abort_flag, st, limit);
 }
 
-// Shared-memory plan: two resident buffers when that still leaves two ring slots, else one;
-// then as many ring slots (up to max_slots) as fit in the 227 KB opt-in limit.
+// Shared-memory plan: as many ring slots (up to MAX_SLOTS) as fit in the 227 KB opt-in limit
+// beside two resident buffers (the next unit's operand loads during this one), or beside one
+// where two would leave fewer: with four K-blocks per tile two slots kept only half a tile in
+// flight, and the threshold kernel waited for its copies a third of the time.
 TcLayout make_layout(uint32_t res_bytes, uint32_t slot_bytes, uint32_t aux_bytes, int max_slots) {
     TcLayout L{};
     aux_bytes = (aux_bytes + 1023u) & ~1023u;
     const uint32_t fixed = 1024u + aux_bytes + 1024u;  // align slack + barriers
-    L.nres = (fixed + 2u * res_bytes + 2u * slot_bytes <= (uint32_t)SMEM_LIMIT) ? 2 : 1;
-    int slots = max_slots;
-    while (slots > 1 && fixed + L.nres * res_bytes + slots * slot_bytes > (uint32_t)SMEM_LIMIT) --slots;
+    auto fit = [&](uint32_t nres) {
+        const uint32_t used = fixed + nres * res_bytes;
+        const int n = used >= (uint32_t)SMEM_LIMIT ? 0 : (int)(((uint32_t)SMEM_LIMIT - used) / slot_bytes);
+        return n < max_slots ? n : max_slots;
+    };
+    L.nres = fit(2) == fit(1) ? 2 : 1;
+    const int slots = fit((uint32_t)L.nres);
     L.slots = slots;
     L.res_bytes = res_bytes;
     L.slot_bytes = slot_bytes;

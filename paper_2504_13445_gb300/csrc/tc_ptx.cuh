@@ -66,6 +66,37 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return true;
 }
 
+// The same wait on a barrier given by its shared-memory address.
+__device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0u;
+}
+
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort, DevStatus* st) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait_at(bar, parity)) {
+        if (*abort) return false;
+        if (clock64() - t0 > RKM_WAIT_CYCLES) {
+            *abort = 1;
+            st->timeout = 1u;
+            return false;
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ bool mbar_wait_at(uint32_t bar, uint32_t parity, volatile int* abort, DevStatus* st) {
+    if (mbar_try_wait_at(bar, parity)) return true;
+    return mbar_wait_slow(bar, parity, abort, st);
+}
+
 // ---- TMA ------------------------------------------------------------------------
 
 // 2-D tiled load of box {x .. x+box0, y .. y+box1} into shared memory, completing on bar.
@@ -133,6 +164,47 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint6
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+
+// The four MMAs of one K-block (128 bytes of every row): descriptors advance by 32 bytes.  alo / blo
+// are the low words of the operands' descriptors (sdesc_lo); `fresh` drops the accumulator's old
+// content.  One statement, with the 64-bit descriptors put together in it.
+template <bool FP8>
+__device__ __forceinline__ void tc_mma_kblock(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc, bool fresh) {
+    constexpr uint32_t HI = (1024u >> 4) | (1u << 14) | (2u << 29);  // high word of sdesc_sw128
+#define RKM_KBLOCK(KIND)                                                        \
+    asm volatile(                                                               \
+        "{\n\t.reg .pred p;\n\t.reg .b32 a, b;\n\t.reg .b64 x, y;\n\t"          \
+        "setp.eq.u32 p, %4, 0;\n\t"                                             \
+        "mov.b64 x, {%1, %5};\n\tmov.b64 y, {%2, %5};\n\t"                      \
+        "tcgen05.mma.cta_group::1." KIND " [%0], x, y, %3, p;\n\t"              \
+        "add.u32 a, %1, 2;\n\tadd.u32 b, %2, 2;\n\t"                            \
+        "mov.b64 x, {a, %5};\n\tmov.b64 y, {b, %5};\n\t"                        \
+        "tcgen05.mma.cta_group::1." KIND " [%0], x, y, %3, 1;\n\t"              \
+        "add.u32 a, %1, 4;\n\tadd.u32 b, %2, 4;\n\t"                            \
+        "mov.b64 x, {a, %5};\n\tmov.b64 y, {b, %5};\n\t"                        \
+        "tcgen05.mma.cta_group::1." KIND " [%0], x, y, %3, 1;\n\t"              \
+        "add.u32 a, %1, 6;\n\tadd.u32 b, %2, 6;\n\t"                            \
+        "mov.b64 x, {a, %5};\n\tmov.b64 y, {b, %5};\n\t"                        \
+        "tcgen05.mma.cta_group::1." KIND " [%0], x, y, %3, 1;\n\t}\n" ::"r"(d_tmem), \
+        "r"(alo), "r"(blo), "r"(idesc), "r"((uint32_t)fresh), "r"(HI)            \
+        : "memory")
+    if constexpr (FP8) RKM_KBLOCK("kind::f8f6f4");
+    else RKM_KBLOCK("kind::f16");
+#undef RKM_KBLOCK
+}
+
+// True in one lane of a full warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0u;
+}
+
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+
+__device__ __forceinline__ void tc_commit_at(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // Instruction descriptor of kind::f8f6f4 with A = B = E4M3 (format code 0 in bits 7-9 and
