@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SimtSmem& sm = *reinterpret_cast<SimtSmem*>(smem_raw);
     int* cnt_s = reinterpret_cast<int*>(smem_raw + sizeof(SimtSmem));  // [BI_SIMT]
+    BandStage stage{reinterpret_cast<int2*>(cnt_s + BI_SIMT) + (threadIdx.x >> 5) * BAND_STAGE, 0};
     __shared__ unsigned s_unit;
     const float* A = static_cast<const float*>(a.A);
     const float* B = static_cast<const float*>(a.B);
@@ -178,7 +179,10 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
         __syncthreads();
         const unsigned w = s_unit;
         __syncthreads();
-        if (w >= total) break;
+        if (w >= total) {
+            if (t < BU) band_flush(stage, a.band, a.band_cap, a.st);
+            break;
+        }
         int T;
         int64_t ut0, ut1;
         decode_count_unit(a, w, T, ut0, ut1);
@@ -204,9 +208,10 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
                 for (int c0 = 0; c0 < BI_SIMT; c0 += 32) {
                     float v[32];
                     load_row_chunk(sm, t, c0, v);
-                    count_chunk(v, active, c0, pos0 + c0, a.m, hi_t, lo_t, cnt_s, u_orig, a.band,
+                    count_chunk(v, active, c0, pos0 + c0, a.m, hi_t, lo_t, cnt_s, u_orig, stage, a.band,
                                 a.band_cap, a.st);
                 }
+                if (stage.n > BAND_STAGE / 2) band_flush(stage, a.band, a.band_cap, a.st);
             }
             __syncthreads();
         }
@@ -232,7 +237,7 @@ void launch_threshold_simt(const ThresholdArgs& a, cudaStream_t s) {
 }
 
 void launch_count_simt(const CountArgs& a, cudaStream_t s) {
-    const size_t smem = sizeof(SimtSmem) + BI_SIMT * sizeof(int);
+    const size_t smem = sizeof(SimtSmem) + BI_SIMT * sizeof(int) + (BU / 32) * BAND_STAGE * sizeof(int2);
     cudaFuncSetAttribute(k_count_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     note_launch();
     k_count_simt<<<a.num_sms, SIMT_THREADS, smem, s>>>(a);

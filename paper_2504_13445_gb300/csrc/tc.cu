@@ -718,46 +718,61 @@ struct CountSet {
     __device__ __forceinline__ const CountArgs& args(int i) const { return MULTI ? inst[i].a : a0; }
     __device__ __forceinline__ const CUtensorMap* mapA(int i) const { return MULTI ? &inst[i].tmA : mA0; }
     __device__ __forceinline__ const CUtensorMap* mapB(int i) const { return MULTI ? &inst[i].tmB : mB0; }
-    // Global unit w -> problem i, item tile T and user tiles [ut0, ut1) of that problem.
-    __device__ __forceinline__ void decode(long long w, int& i, int& T, int64_t& ut0, int64_t& ut1) const {
-        i = MULTI ? count_instance(inst, count, w) : 0;
-        const long long first = MULTI ? inst[i].unit_begin : 0;
-        decode_count_unit(args(i), (unsigned)(w - first), T, ut0, ut1);
+};
+
+// The counting units of one CTA in order (w = blockIdx.x, blockIdx.x + gridDim.x, ...): problem i,
+// item tile T, user tiles [ut0, ut1).  Units are tile-major, so the next one lies in the same tile
+// or mostly in the one after it: two reads where a binary search over the tiles' first units
+// takes one dependent read per halving (about 2,700 cycles at 390 tiles, in which the MMA issuer
+// and the epilogue stood still once per unit).
+template <bool MULTI>
+struct UnitWalk {
+    const CountSet<MULTI>& cs;
+    const long long total;
+    long long w;
+    int i = 0, T = 0;
+    int ut0 = 0, ut1 = 0;
+    int lo = -1, all = 0;       // tile of the problem's list (T - t_begin); its user tiles
+    unsigned u0 = 0, u1 = 0;    // its units [u0, u1)
+    long long first = 0, last;  // the problem's units in the launch
+
+    __device__ __forceinline__ UnitWalk(const CountSet<MULTI>& cs_, long long total_)
+        : cs(cs_), total(total_), w((long long)blockIdx.x - (long long)gridDim.x), last(MULTI ? 0 : total_) {}
+
+    __device__ __forceinline__ bool next() {
+        w += gridDim.x;
+        if (w >= total) return false;
+        if (MULTI && w >= last) {
+            i = count_instance(cs.inst, cs.count, w);
+            first = cs.inst[i].unit_begin;
+            last = i + 1 < cs.count ? cs.inst[i + 1].unit_begin : total;
+            lo = -1;
+        }
+        const CountArgs& a = cs.args(i);
+        const unsigned lw = (unsigned)(w - first);
+        if (lo < 0 || lw >= u1) {
+            if (lo >= 0) {
+                u0 = u1;
+                u1 = a.unit_off[++lo + 1];
+            }
+            if (lo < 0 || lw >= u1) {
+                int hi = a.st->t_end - a.t_begin;  // unit_off has hi + 1 entries
+                lo = lo < 0 ? 0 : lo;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (a.unit_off[mid] <= lw) lo = mid; else hi = mid;
+                }
+                u0 = a.unit_off[lo];
+                u1 = a.unit_off[lo + 1];
+            }
+            T = a.t_begin + lo;
+            all = (int)(((int64_t)a.nprefix[T] + BU - 1) / BU);
+        }
+        ut0 = (int)(lw - u0) * a.group;
+        ut1 = ut0 + a.group < all ? ut0 + a.group : all;
+        return true;
     }
 };
-
-// Position in a CTA's sequence of counting tiles: unit w (problem i, item tile T), user tile
-// ut of [ut0, ut1).  Units are taken as blockIdx.x, blockIdx.x + gridDim.x, ...
-struct TileCursor {
-    long long w;
-    int i, T;
-    int64_t ut, ut1;
-    bool valid;
-};
-
-template <bool MULTI>
-__device__ __forceinline__ void cursor_unit(const CountSet<MULTI>& cs, long long total, TileCursor& c) {
-    c.valid = c.w < total;
-    if (!c.valid) return;
-    int64_t ut0;
-    cs.decode(c.w, c.i, c.T, ut0, c.ut1);
-    c.ut = ut0;
-}
-
-template <bool MULTI>
-__device__ __forceinline__ void cursor_first(const CountSet<MULTI>& cs, long long total, TileCursor& c) {
-    c.w = blockIdx.x;
-    cursor_unit(cs, total, c);
-}
-
-// Every unit holds at least one user tile, so one step never skips a unit.
-template <bool MULTI>
-__device__ __forceinline__ void cursor_next(const CountSet<MULTI>& cs, long long total, TileCursor& c) {
-    if (!c.valid) return;
-    if (++c.ut < c.ut1) return;
-    c.w += gridDim.x;
-    cursor_unit(cs, total, c);
-}
 
 // Add a warp's per-item counters of the CW columns starting at pos0 to the global counts.
 template <int CW>
@@ -825,10 +840,9 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             bool ok = true;
             int last_i = -1;
             unsigned long long pairs = 0;
-            for (long long w = blockIdx.x; w < total && ok; w += gridDim.x) {
-                int i, T;
-                int64_t ut0, ut1;
-                cs.decode(w, i, T, ut0, ut1);
+            UnitWalk<MULTI> wk(cs, total);
+            while (ok && wk.next()) {
+                const int i = wk.i;
                 const CountArgs& a = cs.args(i);
                 if (i != last_i) {
                     if (pairs) atomicAdd(&cs.args(last_i).st->pairs_evaluated, pairs);
@@ -845,16 +859,16 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                 uint8_t* dst = sB + rb * L.res_bytes;
                 mbar_expect_tx(&B->res_full[rb], KB * KB_BYTES_I);
                 for (int kb = 0; kb < KB; ++kb)
-                    tma_load_2d(dst + kb * KB_BYTES_I, mB, &B->res_full[rb], kb * Op::KELEMS, T * BI_TC);
+                    tma_load_2d(dst + kb * KB_BYTES_I, mB, &B->res_full[rb], kb * Op::KELEMS, wk.T * BI_TC);
                 ++res_loads;
-                for (int64_t ut = ut0; ut < ut1 && ok; ++ut) {
+                for (int ut = wk.ut0; ut < wk.ut1 && ok; ++ut) {
                     for (int kb = 0; kb < KB; ++kb) {
                         if (!mbar_wait(&B->empty[slot], ph ^ 1u, abort, st0)) {
                             ok = false;
                             break;
                         }
                         mbar_expect_tx(&B->full[slot], KB_BYTES_U);
-                        tma_load_2d(ring + slot * KB_BYTES_U, mA, &B->full[slot], kb * Op::KELEMS, (int)(ut * BU));
+                        tma_load_2d(ring + slot * KB_BYTES_U, mA, &B->full[slot], kb * Op::KELEMS, ut * BU);
                         ++issued[slot];
                         if (++slot == S) {
                             slot = 0;
@@ -862,8 +876,8 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                         }
                     }
                 }
-                const int64_t uend = (ut1 * BU < a.n) ? ut1 * BU : a.n;
-                if (ut1 > ut0) pairs += (unsigned long long)(uend - ut0 * BU) * BI_TC;
+                const int64_t uend = ((int64_t)wk.ut1 * BU < a.n) ? (int64_t)wk.ut1 * BU : a.n;
+                pairs += (unsigned long long)(uend - (int64_t)wk.ut0 * BU) * BI_TC;
             }
             if (pairs && last_i >= 0) atomicAdd(&cs.args(last_i).st->pairs_evaluated, pairs);
             for (int s = 0; s < S; ++s)
@@ -876,13 +890,11 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
     } else if (warp == 1) {
         Issuer q(B, ring, sB, tmem, Op::idesc());
         int iter = 0;
-        for (long long w = blockIdx.x; w < total; w += gridDim.x, ++iter) {
-            int i, T;
-            int64_t ut0, ut1;
-            cs.decode(w, i, T, ut0, ut1);
+        UnitWalk<MULTI> wk(cs, total);
+        for (; wk.next(); ++iter) {
             const int rb = iter % L.nres;
             if (!q.wait(smem_u32(&B->res_full[rb]), (iter / L.nres) & 1, st0)) break;
-            if (!q.template unit<FP8, true, false>(B, S, (int)(ut1 - ut0), cs.args(i).dp >> Op::KSHIFT,
+            if (!q.template unit<FP8, true, false>(B, S, wk.ut1 - wk.ut0, cs.args(wk.i).dp >> Op::KSHIFT,
                                                    q.reslo + (uint32_t)rb * (L.res_bytes >> 4), NG, st0))
                 break;
             if (elect_one()) tc_commit(&B->res_empty[rb]);
@@ -902,87 +914,91 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
         const int r = q * 32 + lane;
         int* cw = cnt_all + ew * CW;  // this warp's per-item member counters (its CW columns)
         for (int c = lane; c < CW; c += 32) cw[c] = 0;
+        BandStage stage{reinterpret_cast<int2*>(cnt_all + 4 * NG * CW) + ew * BAND_STAGE, 0};
         __syncwarp();
-        // This group consumes global tiles h, h+2, h+4, ... of the CTA's sequence.  `cur` is
-        // the current one, `nxt` the one after it, whose per-user record is loaded one tile
-        // ahead so that its latency hides behind the current tile.
-        TileCursor cur;
-        cursor_first(cs, total, cur);
-        if (h == 1) cursor_next(cs, total, cur);
-        TileCursor nxt = cur;
-        cursor_next(cs, total, nxt);
-        cursor_next(cs, total, nxt);
-        UserMeta um_cur{}, um_nxt{};
-        if (cur.valid && cur.ut * BU + r < cs.args(cur.i).n) um_cur = cs.args(cur.i).meta[cur.ut * BU + r];
-        uint32_t use = 0;
+        // This group consumes every other tile of the CTA's sequence (those of parity h).  The
+        // per-user record of its next tile is loaded one tile ahead, so that its latency hides
+        // behind the current one; a unit's first is loaded in place.
+        UnitWalk<MULTI> wk(cs, total);
+        uint32_t use = 0, seen = 0;  // own tiles done; parity of the tiles before this unit
         int curT = -1, curI = -1;
         float pnh = 0.f, pd = 0.f;
         int te = 0;
         CountHot hot = count_hot(cs.args(0));
-        while (cur.valid) {
-            if (nxt.valid && nxt.ut * BU + r < cs.args(nxt.i).n) um_nxt = cs.args(nxt.i).meta[nxt.ut * BU + r];
-            if (cur.T != curT || cur.i != curI) {
+        bool ok = true;
+        while (ok && wk.next()) {
+            if (wk.T != curT || (MULTI && wk.i != curI)) {
                 if (curT >= 0) flush_counts<CW>(cw, lane, curT * BI_TC + cg, hot.m, hot.counts);
-                if (MULTI && cur.i != curI) hot = count_hot(cs.args(cur.i));
-                const CountArgs& a = cs.args(cur.i);
-                curT = cur.T;
-                curI = cur.i;
-                pnh = a.thmax[cur.T];
-                pd = a.tdel[cur.T];
-                if constexpr (FP8) te = a.texp[cur.T];
-            }
-            if (!mbar_wait(&B->tfull[h], use & 1u, abort, st0)) break;
-            __syncwarp();
-            tc_fence_after();
-            const int64_t us = cur.ut * BU + r;
-            const bool active = us < hot.n;
-            float hi_t = 0.f, lo_t = 0.f;
-            int u_orig = 0;
-            const float f = (FP8 && active) ? pow2i(fp8_exp(um_cur.uexp) + te - 16) : 1.f;  // descale of the FP8 product
-            if (active) {
-                const float E = err_bound(hot.cacc, hot.eabs, um_cur.un, um_cur.unh, um_cur.ud, pnh, pd);
-                hi_t = __fadd_ru(um_cur.tau_hi, E);
-                lo_t = __fsub_rd(um_cur.tau_lo, E);
-                u_orig = um_cur.uorig;
-            }
-            const int pos0 = cur.T * BI_TC + cg;
-            const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)h * BI_TC + cg;
-            uint32_t ra[32], rb[32];
-            // One vote per 64-column pair on the row maxima the two loads return, as in the
-            // threshold epilogue.
-#pragma unroll 1
-            for (int c0 = 0; c0 < CW; c0 += 64) {
-                __syncwarp();
-                float ma, mb;
-                tmem_ld32_max_issue(tb + c0, ra, ma);
-                tmem_ld32_max_issue(tb + c0 + 32, rb, mb);
-                tmem_wait_bind_max(ra, ma);
-                tmem_wait_bind_max(rb, mb);
-                const float mx = FP8 ? fmaxf(ma, mb) * f : fmaxf(ma, mb);
-                if (__any_sync(0xffffffffu, active && mx >= lo_t)) {
-                    float va[32], vb[32];
-                    as_floats(ra, va);
-                    as_floats(rb, vb);
-                    if constexpr (FP8) {
-                        scale_values(va, f);
-                        scale_values(vb, f);
-                    }
-                    count_chunk(va, active, c0, pos0 + c0, hot.m, hi_t, lo_t, cw, u_orig, hot.band,
-                                hot.band_cap, hot.st);
-                    count_chunk(vb, active, c0 + 32, pos0 + c0 + 32, hot.m, hi_t, lo_t, cw, u_orig, hot.band,
-                                hot.band_cap, hot.st);
+                if (MULTI && wk.i != curI) {
+                    band_flush(stage, hot.band, hot.band_cap, hot.st);
+                    hot = count_hot(cs.args(wk.i));
                 }
+                const CountArgs& a = cs.args(wk.i);
+                curT = wk.T;
+                curI = wk.i;
+                pnh = a.thmax[curT];
+                pd = a.tdel[curT];
+                if constexpr (FP8) te = a.texp[curT];
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&B->tempty[h]);
-            ++use;
-            cur = nxt;
-            um_cur = um_nxt;
-            cursor_next(cs, total, nxt);
-            cursor_next(cs, total, nxt);
+            const UserMeta* meta = cs.args(wk.i).meta + r;
+            const int64_t left = hot.n - r;  // this row has a user in tile ut while BU * ut < left
+            int ut = wk.ut0 + (int)((seen ^ (uint32_t)h) & 1u);
+            seen += (uint32_t)(wk.ut1 - wk.ut0);
+            UserMeta um{}, um_nxt{};
+            if (ut < wk.ut1 && (int64_t)ut * BU < left) um = meta[(int64_t)ut * BU];
+            const int pos0 = curT * BI_TC + cg;
+            for (; ut < wk.ut1; ut += 2, ++use) {
+                if (ut + 2 < wk.ut1 && (int64_t)(ut + 2) * BU < left) um_nxt = meta[(int64_t)(ut + 2) * BU];
+                const bool active = (int64_t)ut * BU < left;
+                float hi_t = 0.f, lo_t = 0.f;
+                const float f = (FP8 && active) ? pow2i(fp8_exp(um.uexp) + te - 16) : 1.f;  // descale of the FP8 product
+                if (active) {
+                    const float E = err_bound(hot.cacc, hot.eabs, um.un, um.unh, um.ud, pnh, pd);
+                    hi_t = __fadd_ru(um.tau_hi, E);
+                    lo_t = __fsub_rd(um.tau_lo, E);
+                }
+                if (!mbar_wait(&B->tfull[h], use & 1u, abort, st0)) {
+                    ok = false;
+                    break;
+                }
+                __syncwarp();
+                tc_fence_after();
+                const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)h * BI_TC + cg;
+                uint32_t ra[32], rb[32];
+                // One vote per 64-column pair on the row maxima the two loads return, as in the
+                // threshold epilogue.
+#pragma unroll 1
+                for (int c0 = 0; c0 < CW; c0 += 64) {
+                    __syncwarp();
+                    float ma, mb;
+                    tmem_ld32_max_issue(tb + c0, ra, ma);
+                    tmem_ld32_max_issue(tb + c0 + 32, rb, mb);
+                    tmem_wait_bind_max(ra, ma);
+                    tmem_wait_bind_max(rb, mb);
+                    const float mx = FP8 ? fmaxf(ma, mb) * f : fmaxf(ma, mb);
+                    if (__any_sync(0xffffffffu, active && mx >= lo_t)) {
+                        float va[32], vb[32];
+                        as_floats(ra, va);
+                        as_floats(rb, vb);
+                        if constexpr (FP8) {
+                            scale_values(va, f);
+                            scale_values(vb, f);
+                        }
+                        count_chunk(va, active, c0, pos0 + c0, hot.m, hi_t, lo_t, cw, um.uorig, stage, hot.band,
+                                    hot.band_cap, hot.st);
+                        count_chunk(vb, active, c0 + 32, pos0 + c0 + 32, hot.m, hi_t, lo_t, cw, um.uorig, stage,
+                                    hot.band, hot.band_cap, hot.st);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&B->tempty[h]);
+                if (stage.n > BAND_STAGE / 2) band_flush(stage, hot.band, hot.band_cap, hot.st);
+                um = um_nxt;
+            }
         }
         if (curT >= 0) flush_counts<CW>(cw, lane, curT * BI_TC + cg, hot.m, hot.counts);
+        band_flush(stage, hot.band, hot.band_cap, hot.st);
     }
     teardown(B, warp);
 }
@@ -1288,8 +1304,10 @@ template <bool FP8, int NG, bool MULTI>
 void launch_count_ng(const CountArgs& a0, const CUtensorMap& mA, const CUtensorMap& mB, const CountInstance* inst,
                      int count, const unsigned long long* total, int max_dp, int grid, cudaStream_t s) {
     const int KB = FP8 ? max_dp / 128 : max_dp / 64;
-    // per-warp member counters: 4 NG warps x (512 / NG) columns
-    const TcLayout L = make_layout(KB * KB_BYTES_I, KB_BYTES_U, 4u * NG * (2u * BI_TC / NG) * 4u, MAX_SLOTS);
+    // per-warp member counters (4 NG warps x 512 / NG columns) and staged band pairs
+    const TcLayout L = make_layout(KB * KB_BYTES_I, KB_BYTES_U,
+                                   4u * NG * (2u * BI_TC / NG) * 4u + 4u * NG * BAND_STAGE * (uint32_t)sizeof(int2),
+                                   MAX_SLOTS);
     cudaFuncSetAttribute(k_count_tc<FP8, NG, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
     k_count_tc<FP8, NG, MULTI><<<grid, tc_threads(NG), L.bytes, s>>>(a0, mA, mB, inst, count, total, L);
 }
