@@ -67,7 +67,7 @@ struct __align__(16) UserMeta {
 };
 
 // Candidate of the threshold pass: an upper bound of u.p and the item's sorted position.
-struct Cand {
+struct __align__(8) Cand {
     float ub;
     int pos;
 };

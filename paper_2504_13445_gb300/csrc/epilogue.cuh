@@ -59,7 +59,8 @@ struct SelState {
     unsigned long long* pub;  // where this group publishes its bound for the other (null: none)
     unsigned tag;             // user tile the published bound belongs to
     int defer;   // 1: hits only record candidates; sel_merge_tile admits them at the tile's end
-    int mark;    // first candidate recorded in the current tile (-1 after a compaction in it)
+    int mark;    // first candidate not yet offered to the heap (-1 after a compaction)
+    float Em;    // largest error bound of the tiles since
 };
 
 // The best lower bound of tau_u this group knows.
@@ -143,35 +144,50 @@ __device__ __forceinline__ float cand_lower(float ub, float E) {
     return __fsub_rd(__fsub_rd(__fsub_rd(ub, E), E), d);
 }
 
-// Deferred admissions: the lower bounds of the candidates recorded since the tile started
-// enter the heap at the tile's end, with every lane of the warp stepping through its own
-// list together (the heap is built at most once per lane, in one place, instead of at the
-// hit that completes it).  Skipping admissions is sound (see sel_insert), so a tile whose
-// entries a compaction moved admits nothing.
-__device__ __forceinline__ void sel_merge_tile(SelState& s, const Cand* mycand, float* heap, int t, int k, float E,
-                                               bool active) {
-    const int j0 = s.mark, j1 = s.cnt;
+// Deferred admissions: the lower bounds of the candidates recorded since the last call enter the
+// heap with every lane of the warp stepping through its own list together (the heap is built at
+// most once per lane, in one place, instead of at the hit that completes it).  Candidates are read
+// back four at a time, so that a step waits for one read instead of four.  Skipping admissions
+// is sound (see sel_insert), so a list that a compaction moved admits nothing.
+__device__ __forceinline__ void sel_merge(SelState& s, const Cand* mycand, float* heap, int t, int k, bool active) {
+    const float E = s.Em;
+    int j = s.mark;
+    const int j1 = s.cnt;
     s.mark = s.cnt;
-    if (!active || j0 < 0 || j0 >= j1) return;
+    s.Em = 0.f;
+    if (!active || j < 0 || j >= j1) return;
     const float L0 = sel_bound(s);
-    int j = j0;
     bool filled = false;
-    for (; j < j1 && s.hn < k; ++j) {
-        const float lb = cand_lower(mycand[j].ub, E);
-        if (lb > L0) {
-            heap[s.hn * BU + t] = lb;
-            if (++s.hn == k) filled = true;
+    while (j < j1 && s.hn < k) {
+        float ub[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ub[i] = j + i < j1 ? mycand[j + i].ub : -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (s.hn == k || j >= j1) break;
+            const float lb = cand_lower(ub[i], E);
+            if (lb > L0) {
+                heap[s.hn * BU + t] = lb;
+                if (++s.hn == k) filled = true;
+            }
+            ++j;
         }
     }
     if (filled) {
         heapify(heap, t, k);
         s.L = heap[t];
     }
-    for (; j < j1; ++j) {
-        const float lb = cand_lower(mycand[j].ub, E);
-        if (lb > sel_bound(s)) {
-            heap_replace_root(heap, t, k, lb);
-            s.L = heap[t];
+    while (j < j1) {
+        float ub[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ub[i] = j + i < j1 ? mycand[j + i].ub : -INFINITY;
+#pragma unroll 1
+        for (int i = 0; i < 4 && j < j1; ++i, ++j) {
+            const float lb = cand_lower(i == 0 ? ub[0] : i == 1 ? ub[1] : i == 2 ? ub[2] : ub[3], E);
+            if (lb > sel_bound(s)) {
+                heap_replace_root(heap, t, k, lb);
+                s.L = heap[t];
+            }
         }
     }
     if (s.hn == k && s.pub) publish_bound(s.pub, s.tag, fmaxf(s.L, s.Lw));
@@ -226,6 +242,29 @@ __device__ __forceinline__ void sel_chunk(const float (&v)[32], bool active, int
     group_max8(v, g);
     const float mx = fmax3f(g[0], g[1], fmaxf(g[2], g[3]));
     if (!__any_sync(0xffffffffu, active && mx >= s.thr)) return;
+    if (s.defer && pos0 + 32 <= m && !__any_sync(0xffffffffu, active && s.cnt + 32 > cap)) {
+        // Room for the whole chunk and no column past the items: the columns of each 8-column
+        // group with a hit are compared and stored in place, without a branch per hit.
+        Cand* p = mycand + s.cnt;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool hq = active && g[q] >= s.thr;
+            if (!__any_sync(0xffffffffu, hq)) continue;
+            const float thr = hq ? s.thr : INFINITY;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float x = v[8 * q + j];
+                if (hq && x >= thr) {
+                    Cand c;
+                    c.ub = __fadd_ru(x, E);
+                    c.pos = pos0 + 8 * q + j;
+                    *p++ = c;
+                }
+            }
+        }
+        s.cnt = (int)(p - mycand);
+        return;
+    }
     unsigned mask = hit_mask(v, g, active, s.thr);
     while (mask) {
         const int c = __ffs(mask) - 1;
@@ -301,6 +340,23 @@ __device__ __forceinline__ void count_chunk(const float (&v)[32], bool active, i
     }
 }
 
+// Bitonic network over N registers in descending order, from merges of SIZE on.
+template <int N, int SIZE, int STRIDE = SIZE / 2>
+__device__ __forceinline__ void sort_desc(float (&v)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int j = i ^ STRIDE;
+        if (j > i) {
+            const float hi = fmaxf(v[i], v[j]), lo = fminf(v[i], v[j]);
+            const bool desc = (i & SIZE) == 0;
+            v[i] = desc ? hi : lo;
+            v[j] = desc ? lo : hi;
+        }
+    }
+    if constexpr (STRIDE > 1) sort_desc<N, SIZE, STRIDE / 2>(v);
+    else if constexpr (SIZE < N) sort_desc<N, SIZE * 2>(v);
+}
+
 // Warm-start bound from COLS columns of one accumulator row held in TMEM: the maxima of
 // the NG column groups of width COLS/NG, sorted by a bitonic network in registers; the k-th
 // largest (k <= NG) minus E bounds tau_u from below, because k distinct items reach it.
@@ -322,22 +378,7 @@ __device__ __forceinline__ float warm_bound(LoadChunk load, int pos0, int64_t m,
             g[(c0 / GW) + q] = x;
         }
     }
-#pragma unroll
-    for (int size = 2; size <= NG; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-#pragma unroll
-            for (int i = 0; i < NG; ++i) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const float hi = fmaxf(g[i], g[j]), lo = fminf(g[i], g[j]);
-                    const bool desc = (i & size) == 0;
-                    g[i] = desc ? hi : lo;
-                    g[j] = desc ? lo : hi;
-                }
-            }
-        }
-    }
+    sort_desc<NG, 2>(g);
     float kth = -INFINITY;
 #pragma unroll
     for (int j = 0; j < NG; ++j)

@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_threshold_simt(ThresholdArg
         s.tag = 0u;
         s.defer = 0;
         s.mark = 0;
+        s.Em = 0.f;
         float un = 0.f, unh = 0.f, ud = 0.f;
         Cand* mycand = nullptr;
         if (owner) {

@@ -37,6 +37,9 @@ namespace {
 // Threads of a product kernel with NG epilogue warpgroups.
 constexpr int tc_threads(int ng) { return 64 + 128 * ng; }
 constexpr int MAX_SLOTS = 4;
+constexpr int STOP_AHEAD = 8;   // tiles between the stop's test and the tile it tests
+constexpr int MERGE_TILES = 8;  // own tiles, or
+constexpr int MERGE_HITS = 2;   // candidates of one row, between admissions to the heap
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t KB_BYTES_U = 128 * 128;  // one K-block (128 bytes: 64 BF16 / 128 FP8) of 128 user rows
 constexpr uint32_t KB_BYTES_I = 256 * 128;  // one K-block of 256 item rows
@@ -287,27 +290,6 @@ __device__ __forceinline__ int unit_instance(const TcInstance* inst, int count, 
 // Seed pass: values per row and warpgroup, and its shared exchange buffer [SEED_SLOTS][BU].
 constexpr int SEED_SLOTS = 64;
 
-// v sorted in descending order (bitonic network over registers); from: first merge size.
-template <int FROM>
-__device__ __forceinline__ void sort64_desc(float (&v)[SEED_SLOTS]) {
-#pragma unroll
-    for (int size = FROM; size <= SEED_SLOTS; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-#pragma unroll
-            for (int i = 0; i < SEED_SLOTS; ++i) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const float hi = fmaxf(v[i], v[j]), lo = fminf(v[i], v[j]);
-                    const bool desc = (i & size) == 0;
-                    v[i] = desc ? hi : lo;
-                    v[j] = desc ? lo : hi;
-                }
-            }
-        }
-    }
-}
-
 // Threshold pass over one or many independent problems.  Work units are (instance, user
 // tile) pairs numbered consecutively across the instances; CTA b takes units b, b + grid, ...
 // A unit streams every item tile of its instance, so the caller orders the instances by
@@ -488,7 +470,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             }
             if (!ok) break;
             // The 64 largest of both groups' sorted lists are the larger of v[i] and o[63 - i].
-            sort64_desc<2>(v);
+            sort_desc<SEED_SLOTS, 2>(v);
             if (h == 1) {
                 if (!mbar_wait(&B->xempty, xphase ^ 1u, abort, a.st)) break;
 #pragma unroll
@@ -501,7 +483,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                 for (int i = 0; i < SEED_SLOTS; ++i) v[i] = fmaxf(v[i], heaps[(SEED_SLOTS - 1 - i) * BU + r]);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&B->xempty);
-                sort64_desc<SEED_SLOTS>(v);
+                sort_desc<SEED_SLOTS, SEED_SLOTS>(v);
                 float kth = -INFINITY;
 #pragma unroll
                 for (int i = 0; i < SEED_SLOTS; ++i)
@@ -524,13 +506,19 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             const TcInstance& I = inst[unit_instance(inst, count, w)];
             const ThresholdArgs& a = I.a;
             const long long ut = w - I.unit_begin;
-            const int item_tiles = (int)((a.m + BI_TC - 1) / BI_TC);
+            // The fields used on every tile, in registers: read through the descriptor they were
+            // loaded again after every barrier and TMEM access.
+            const int m = (int)a.m, k = a.k, cap = a.cap;
+            const int item_tiles = (int)(((int64_t)m + BI_TC - 1) / BI_TC);
+            const float cacc = a.cacc, eabs = a.eabs;
+            const float *const tmax = a.tmax, *const thmax = a.thmax, *const tdel = a.tdel;
+            DevStatus* const st = a.st;
             const int64_t u = ut * BU + r;
             // The candidate lists have one segment per warpgroup; an instance prepared for
             // another group count is a host bug: flag it and write nothing.
             if (a.nseg != NG && lane == 0 && q == 0) a.st->internal_error = 1u;
             const bool active = u < a.n && a.nseg == NG;
-            for (int j = 0; j < a.k; ++j) heap[j * BU + r] = -INFINITY;
+            for (int j = 0; j < k; ++j) heap[j * BU + r] = -INFINITY;
             SelState s;
             s.L = -INFINITY;
             s.hn = 0;
@@ -542,9 +530,10 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             s.tag = (unsigned)w;
             s.defer = 1;
             s.mark = 0;
+            s.Em = 0.f;
             bool warm = a.lfin_seed != nullptr;  // warm start done for this unit (or seeded)
-            int fb = item_tiles;       // first tile after the last searched one whose
-            float bnd_fb = -INFINITY;  // ||u|| max||p|| is below bnd_fb (see the stop below)
+            bool stopped = false;       // this warp has published where it may stop
+            int since = 0;              // own tiles since candidates were offered to the heap
             // Packed row u holds original user uo; a seed bound of tau_u (from a pass over the
             // highest-norm items) starts the selector above -inf.
             const int64_t uo = (active && a.uperm) ? (int64_t)a.uperm[u] : u;
@@ -554,14 +543,14 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             const float unh = active ? a.unhat[uo] : 0.f;
             const float ud = active ? a.udel[uo] : 0.f;
             const int ue = (FP8 && active) ? fp8_exp(a.uexp[uo]) : 0;
-            Cand* mycand = a.cand + ((active ? u : 0) * a.nseg + g) * (int64_t)a.cap;
+            Cand* mycand = a.cand + ((active ? u : 0) * a.nseg + g) * (int64_t)cap;
             // This group's first tile of the unit, then every other one: the bound maxima of
             // the next one are loaded while the current one is processed.
             int itn = (int)((tile_j & 1u) == (uint32_t)h ? 0 : 1);
             float thm_next = 0.f, tdl_next = 0.f;
             if (itn < item_tiles) {
-                thm_next = a.thmax[itn];
-                tdl_next = a.tdel[itn];
+                thm_next = thmax[itn];
+                tdl_next = tdel[itn];
             }
             for (int it = 0; it < item_tiles; ++it) {
                 const uint32_t b = tile_j & 1u, use = tile_j >> 1;
@@ -569,10 +558,12 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                 if ((int)b != h) continue;
                 const float thm = thm_next, tdl = tdl_next;
                 if (it + 2 < item_tiles) {
-                    thm_next = a.thmax[it + 2];
-                    tdl_next = a.tdel[it + 2];
+                    thm_next = thmax[it + 2];
+                    tdl_next = tdel[it + 2];
                 }
-                if (!mbar_wait(&B->tfull[b], use & 1u, abort, a.st)) {
+                const bool ahead_ok = it + STOP_AHEAD < item_tiles;
+                const float ahead = ahead_ok ? tmax[it + STOP_AHEAD] : 0.f;
+                if (!mbar_wait(&B->tfull[b], use & 1u, abort, st)) {
                     ok = false;
                     break;
                 }
@@ -591,7 +582,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                     if (mk == 1) ++tile_j;
                     break;
                 }
-                const float E = err_bound(a.cacc, a.eabs, un, unh, ud, thm, tdl);
+                const float E = err_bound(cacc, eabs, un, unh, ud, thm, tdl);
                 const float f = FP8 ? pow2i(ue + a.texp[it] - 16) : 1.f;  // descale of the FP8 product
                 // The other groups' bounds may be stale or from this unit's start (-inf):
                 // any value they held is a valid lower bound of tau_u for the current user.
@@ -613,7 +604,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                         tmem_ld32(tb + c0, v);
                         if constexpr (FP8) scale_values(v, f);
                     };
-                    const float lw = warm_bound<CW / 4, CW>(load, it * BI_TC + cg, a.m, a.k, E);
+                    const float lw = warm_bound<CW / 4, CW>(load, it * BI_TC + cg, m, k, E);
                     s.Lw = active ? lw : -INFINITY;
                     publish_bound(s.pub, s.tag, s.Lw);
                     warm = true;
@@ -644,45 +635,38 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                             scale_values(va, f);
                             scale_values(vb, f);
                         }
-                        sel_chunk(va, active, it * BI_TC + cg + c0, a.m, E, s, mycand, a.cap, heap, r, a.k, a.st);
-                        sel_chunk(vb, active, it * BI_TC + cg + c0 + 32, a.m, E, s, mycand, a.cap, heap, r, a.k,
-                                  a.st);
+                        sel_chunk(va, active, it * BI_TC + cg + c0, m, E, s, mycand, cap, heap, r, k, st);
+                        sel_chunk(vb, active, it * BI_TC + cg + c0 + 32, m, E, s, mycand, cap, heap, r, k, st);
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&B->tempty[b]);
-                // The accumulator is released: admit this tile's candidates while the MMA
-                // computes the next tiles.
-                sel_merge_tile(s, mycand, heap, r, a.k, E, active);
+                // The accumulator is released: admit candidates while the MMA computes the next
+                // tiles.  A round of admissions costs the longest list of the warp, so after the
+                // first tiles, with a fraction of a hit per row and tile, rounds wait for
+                // MERGE_HITS candidates of some row or MERGE_TILES own tiles.
+                s.Em = fmaxf(s.Em, E);
+                if (++since == MERGE_TILES ||
+                    __any_sync(0xffffffffu, active && s.mark >= 0 && s.cnt - s.mark >= MERGE_HITS)) {
+                    sel_merge(s, mycand, heap, r, k, active);
+                    since = 0;
+                }
                 // Algorithm 1's stop by Cauchy-Schwarz: items arrive in descending norm order,
                 // so once ||u|| max||p|| of a tile (rounded up) is below a lower bound of tau_u,
-                // no item of that tile or any later one can reach tau_u or tie it.  Publish how
-                // many leading tiles this warp's users still need.
-                // The first tile below a bound moves back as the bound grows, so the search
-                // is skipped while the bound is unchanged and narrowed to [it + 1, fb] when it
-                // grew; the other groups' bounds can make it drop (a group that has moved on
-                // publishes for its next unit), and then the whole rest is searched.
-                {
+                // no item of that tile or any later one can reach tau_u or tie it.  A warp tests
+                // the tile STOP_AHEAD tiles on (more than the ring and the accumulators hold, so the
+                // producer has not loaded it yet) and publishes its index once none of its users
+                // needs it.  (Searching for the first such tile after every own tile took 450 of
+                // 1,300 cycles per own tile at 2M x 500K.)
+                if (!stopped && ahead_ok) {
                     const float bnd = sel_bound(s);
-                    int need = 0;
-                    if (active) {
-                        if (bnd != bnd_fb || fb < it + 1) {
-                            int lo = it + 1, hi = item_tiles;  // first tile below the bound
-                            if (bnd >= bnd_fb && fb < hi) hi = fb > lo ? fb : lo;
-                            while (lo < hi) {
-                                const int mid = (lo + hi) >> 1;
-                                if (__fmul_ru(un, a.tmax[mid]) < bnd) hi = mid; else lo = mid + 1;
-                            }
-                            fb = lo;
-                            bnd_fb = bnd;
-                        }
-                        need = fb;
+                    if (!__any_sync(0xffffffffu, active && !(__fmul_ru(un, ahead) < bnd))) {
+                        stopped = true;
+                        if (lane == 0)
+                            *reinterpret_cast<volatile unsigned long long*>(&B->need_pub[ew]) =
+                                ((unsigned long long)(unsigned)w << 32) | (unsigned)(it + STOP_AHEAD);
                     }
-                    need = __reduce_max_sync(0xffffffffu, need);
-                    if (lane == 0)
-                        *reinterpret_cast<volatile unsigned long long*>(&B->need_pub[ew]) =
-                            ((unsigned long long)(unsigned)w << 32) | (unsigned)need;
                 }
             }
             if (active) {
