@@ -24,10 +24,14 @@ struct TopnSmem {
     unsigned long long prefix;
     unsigned need;
     unsigned sel_count;
+    int done;
     unsigned long long sel[NMAX_TOPN];
 };
 
-// Top N of positions [0, M) (all threads of the CTA call it).
+// Top N of positions [0, M) (all threads of the CTA call it).  One warp finds each digit by a scan of
+// eight buckets per lane (one thread walking the 256 buckets took 4 us per digit, 32 of the 37 us
+// of a call on 1,000 items), and the select ends at the first digit whose bucket holds exactly
+// the keys still needed: usually the second or third of eight.
 __device__ __forceinline__ void topn_select(TopnSmem& sm, const int* __restrict__ counts,
                                             const int* __restrict__ item_id, int64_t M, int N, int* __restrict__ ids,
                                             int* __restrict__ scores, DevStatus* st) {
@@ -40,6 +44,7 @@ __device__ __forceinline__ void topn_select(TopnSmem& sm, const int* __restrict_
         sm.prefix = 0ull;
         sm.need = (unsigned)N;
         sm.sel_count = 0u;
+        sm.done = 0;
     }
     unsigned long long mask = 0ull;
     for (int shift = 56; shift >= 0; shift -= 8) {
@@ -51,20 +56,43 @@ __device__ __forceinline__ void topn_select(TopnSmem& sm, const int* __restrict_
             if ((key & mask) == prefix) atomicAdd(&sm.hist[(key >> shift) & 255u], 1u);
         }
         __syncthreads();
-        if (t == 0) {
-            unsigned need = sm.need, cum = 0u;
-            int dg = 255;
-            for (; dg > 0; --dg) {
-                if (cum + sm.hist[dg] >= need) break;
-                cum += sm.hist[dg];
+        if (t < 32) {
+            const unsigned need = sm.need;
+            unsigned c[8], sum = 0u;  // digits 255 - 8 t .. 248 - 8 t
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                c[j] = sm.hist[255 - 8 * t - j];
+                sum += c[j];
             }
-            sm.need = need - cum;
-            sm.prefix = prefix | ((unsigned long long)dg << shift);
+            unsigned x = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+                if (t >= o) x += y;
+            }
+            unsigned cum = x - sum;  // keys of larger digits
+            if (cum < need && x >= need) {
+                int j = 0;
+#pragma unroll
+                for (int i = 0; i < 7; ++i) {
+                    if (j == i && cum + c[i] < need) {
+                        cum += c[i];
+                        ++j;
+                    }
+                }
+                unsigned at = c[0];
+#pragma unroll
+                for (int i = 1; i < 8; ++i) at = j == i ? c[i] : at;
+                sm.need = need - cum;
+                sm.prefix = prefix | ((unsigned long long)(255 - 8 * t - j) << shift);
+                sm.done = at == need - cum;
+            }
         }
         mask |= (0xFFull << shift);
         __syncthreads();
+        if (sm.done) break;
     }
-    // sm.prefix is now the N-th largest key; keys are unique, so exactly N keys are >= it.
+    // Exactly N of the (unique) keys are at or above sm.prefix.
     const unsigned long long kth = sm.prefix;
     for (int64_t p = t; p < M; p += TOPN_THREADS) {
         const unsigned long long key = topn_key(counts, item_id, p);
