@@ -795,6 +795,15 @@ rkm_status count_descriptor(const PathShape& ps, int64_t n, const UserOrder& uo,
     return RKM_OK;
 }
 
+// User tiles per counting work unit: the context's (32, or the autotuner's), or fewer where that
+// would leave the SMs less than about 8 units each.  2,000 users x 1,000 items made 4 units of 16
+// tiles (81 us on 4 SMs; 64 units of one tile: 22 us), and 32 candidates against a million users
+// 244 units for 152 SMs.  Smaller units than needed reload the resident item tile more often.
+int unit_tiles(const rkm_ctx* c, int64_t n, int item_tiles) {
+    const int64_t tiles = (n + BU - 1) / BU * item_tiles;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(c->count_group, tiles / ((int64_t)c->num_sms * 8)));
+}
+
 // One counting stage over item tiles [t_begin, t_end) (t_end from the device if t_end_dev).
 rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrder& uo, const ItemSide& it,
                        bool new_items, int t_begin, int t_end, bool t_end_from_dev, const ExactData& x,
@@ -803,10 +812,10 @@ rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrd
     unsigned* unit_off;
     TRY(c->ensure(c->nprefix, std::max<int64_t>(it.tiles, 1), &nprefix));
     TRY(c->ensure(c->unit_off, it.tiles + 2, &unit_off));
-    const int group = c->count_group;  // user tiles per work unit
+    const int group = unit_tiles(c, n, (t_end_from_dev ? (int)it.tiles : t_end) - t_begin);
     Phase ph_count(c, s, RKM_PHASE_COUNT);
     launch_build_units(it.tmax, uo.ucum, t_begin, t_end, t_end_from_dev ? &c->st->t_end : nullptr, BU, group,
-                       nprefix, unit_off, c->st, s);
+                       nprefix, unit_off, (unsigned)c->band_cap, c->st, s);
     CountArgs a{};
     a.A = uo.pack;
     a.B = it.pack;

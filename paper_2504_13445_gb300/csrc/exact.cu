@@ -908,11 +908,6 @@ __global__ void __launch_bounds__(32 * BAND_WARPS, 8)
                gridDim.x * BAND_WARPS, work[w]);
 }
 
-__global__ void k_band_mark(DevStatus* st, unsigned band_cap) {
-    unsigned end = st->band_count;
-    st->band_done = end > band_cap ? band_cap : end;
-}
-
 // Band rescoring of job blockIdx.y (catalogue items: ties at tau_u are decided by t_u).
 __global__ void __launch_bounds__(32 * BAND_WARPS) k_band_rescore_multi(const BatchJob* __restrict__ jobs) {
     __shared__ BandWarp work[BAND_WARPS];
@@ -920,14 +915,6 @@ __global__ void __launch_bounds__(32 * BAND_WARPS) k_band_rescore_multi(const Ba
     const BatchJob& J = jobs[blockIdx.y];
     band_pairs(J.x, J.band, J.band_cap, J.item_perm, J.tau, J.tid, false, J.counts, J.st, blockIdx.x * BAND_WARPS + w,
                gridDim.x * BAND_WARPS, work[w]);
-}
-
-__global__ void k_band_mark_multi(const BatchJob* __restrict__ jobs, int count) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= count) return;
-    DevStatus* st = jobs[j].st;
-    const unsigned end = st->band_count, cap = jobs[j].band_cap;
-    st->band_done = end > cap ? cap : end;
 }
 
 // Zero the counts of job blockIdx.y and its band counters.
@@ -999,8 +986,6 @@ void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap
     (void)m_ids;
     note_launch();
     k_band_rescore<<<1216, 32 * BAND_WARPS, 0, s>>>(x, band, band_cap, item_perm, tau, tid, new_items, counts, st);
-    note_launch();
-    k_band_mark<<<1, 1, 0, s>>>(st, band_cap);
 }
 
 void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users, cudaStream_t s) {
@@ -1013,8 +998,6 @@ void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users
 void launch_band_multi(const BatchJob* jobs, int count, cudaStream_t s) {
     note_launch();
     k_band_rescore_multi<<<dim3(128, (unsigned)count), 32 * BAND_WARPS, 0, s>>>(jobs);
-    note_launch();
-    k_band_mark_multi<<<(count + 127) / 128, 128, 0, s>>>(jobs, count);
 }
 
 void launch_batch_reset(const BatchJob* jobs, int count, int64_t max_m, cudaStream_t s) {

@@ -222,10 +222,11 @@ struct CountArgs {
     DevStatus* st;
     int num_sms;
 };
-// Work list of a counting stage over item tiles [t_begin, t_end or *t_end_dev).
+// Work list of a counting stage over item tiles [t_begin, t_end or *t_end_dev).  The band pairs
+// queued so far (at most band_cap) are marked as rescored: the stage before has been.
 void launch_build_units(const float* tmax, const unsigned* ucum, int t_begin, int t_end,
                         const int* t_end_dev, int tile_users, int group, int* nprefix,
-                        unsigned* unit_off, DevStatus* st, cudaStream_t s);
+                        unsigned* unit_off, unsigned band_cap, DevStatus* st, cudaStream_t s);
 void launch_count_simt(const CountArgs& a, cudaStream_t s);
 
 // One problem of a tensor-core counting launch: its TMA maps (users in ratio order, items
@@ -286,7 +287,7 @@ void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users
 void launch_batch_reset(const BatchJob* jobs, int count, int64_t max_m, cudaStream_t s);
 // Unit lists of counting stage 1 (tiles [0, t0)) or 2 (tiles [t0, st->t_end)) of every problem.
 void launch_build_units_multi(const BatchJob* jobs, int count, int stage, cudaStream_t s);
-// Exact rescoring of every problem's new band pairs, then marks them done.
+// Exact rescoring of every problem's new band pairs.
 void launch_band_multi(const BatchJob* jobs, int count, cudaStream_t s);
 // Top-N of every problem: stage 1 over the first-stage items into top_ids_c0/top_sc_c0,
 // stage 2 over the counted items into ids/top_scores.

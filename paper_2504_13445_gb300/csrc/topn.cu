@@ -182,7 +182,7 @@ __global__ void k_filter_cut_multi(const BatchJob* __restrict__ jobs, int count)
 __device__ __forceinline__ void build_units(const float* __restrict__ tmax, const unsigned* __restrict__ ucum,
                                             int t_begin, int t_end, int tile_users, int group,
                                             int* __restrict__ nprefix, unsigned* __restrict__ unit_off,
-                                            DevStatus* st) {
+                                            unsigned band_cap, DevStatus* st) {
     constexpr int T = 1024;
     __shared__ unsigned part[T];
     const int t = threadIdx.x;
@@ -218,13 +218,17 @@ __device__ __forceinline__ void build_units(const float* __restrict__ tmax, cons
         st->units_total = part[T - 1];
         st->ticket = 0u;
         st->t_end = t_end;
+        const unsigned pushed = st->band_count;
+        st->band_done = pushed < band_cap ? pushed : band_cap;
     }
 }
 
 __global__ void k_build_units(const float* __restrict__ tmax, const unsigned* __restrict__ ucum, int t_begin,
                               int t_end_host, const int* t_end_dev, int tile_users, int group,
-                              int* __restrict__ nprefix, unsigned* __restrict__ unit_off, DevStatus* st) {
-    build_units(tmax, ucum, t_begin, t_end_dev ? *t_end_dev : t_end_host, tile_users, group, nprefix, unit_off, st);
+                              int* __restrict__ nprefix, unsigned* __restrict__ unit_off, unsigned band_cap,
+                              DevStatus* st) {
+    build_units(tmax, ucum, t_begin, t_end_dev ? *t_end_dev : t_end_host, tile_users, group, nprefix, unit_off,
+                band_cap, st);
 }
 
 // Unit lists of job blockIdx.x: stage 1 over tiles [0, t0), stage 2 over [t0, st->t_end).
@@ -232,7 +236,7 @@ __global__ void k_build_units_multi(const BatchJob* __restrict__ jobs, int stage
     const BatchJob& J = jobs[blockIdx.x];
     const int t_begin = stage == 1 ? 0 : J.t0;
     const int t_end = stage == 1 ? J.t0 : J.st->t_end;
-    build_units(J.tmax, J.ucum, t_begin, t_end, BU, J.group, J.nprefix, J.unit_off, J.st);
+    build_units(J.tmax, J.ucum, t_begin, t_end, BU, J.group, J.nprefix, J.unit_off, J.band_cap, J.st);
 }
 
 }  // namespace
@@ -250,11 +254,11 @@ void launch_filter_cut(const int* top_scores_c0, int N, const float* tmax, const
 }
 
 void launch_build_units(const float* tmax, const unsigned* ucum, int t_begin, int t_end, const int* t_end_dev,
-                        int tile_users, int group, int* nprefix, unsigned* unit_off, DevStatus* st,
+                        int tile_users, int group, int* nprefix, unsigned* unit_off, unsigned band_cap, DevStatus* st,
                         cudaStream_t s) {
     note_launch();
     k_build_units<<<1, 1024, 0, s>>>(tmax, ucum, t_begin, t_end, t_end_dev, tile_users, group, nprefix,
-                                     unit_off, st);
+                                     unit_off, band_cap, st);
 }
 
 void launch_topn_multi(const BatchJob* jobs, int count, int stage, cudaStream_t s) {
