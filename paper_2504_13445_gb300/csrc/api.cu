@@ -1754,23 +1754,45 @@ rkm_status batch_enqueue(rkm_ctx* c, const rkm_instance* inst, int count, cudaSt
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
             return instance_cost(inst[x], w[x].ps) > instance_cost(inst[y], w[y].ps);
         });
-        if (c->batch_host_cap < count) {
+        // Descriptors of the main launch, then of the seed pass.
+        if (c->batch_host_cap < 2 * count) {
             if (c->batch_host) cudaFreeHost(c->batch_host);
             c->batch_host = nullptr;
             c->batch_host_cap = 0;
-            CUDA_TRY(cudaMallocHost(&c->batch_host, (size_t)count * sizeof(TcInstance)));
-            c->batch_host_cap = count;
+            CUDA_TRY(cudaMallocHost(&c->batch_host, 2 * (size_t)count * sizeof(TcInstance)));
+            c->batch_host_cap = 2 * count;
         }
         TcInstance* dev;
-        TRY(c->ensure(c->batch_dev, count, &dev));
-        long long units = 0;
+        TRY(c->ensure(c->batch_dev, 2 * (int64_t)count, &dev));
+        // One seed launch for every instance whose size its rule takes.  Users stay in input order
+        // here: the seed order costs each instance a sort and a second pack of its users, six more
+        // launches, which the better stop of a small instance does not pay for.
+        long long units = 0, seed_units = 0;
+        int seeded = 0;
         for (int j = 0; j < count; ++j) {
             const int i = order[j];
-            TRY(threshold_descriptor(w[i].ps, w[i].pl, w[i].it, &c->batch_host[j]));
+            InstWork& x = w[i];
+            const int64_t seeds = c->opts.seed_order ? seed_tiles(x.ps, x.it.tiles, inst[i].k) : 0;
+            if (seeds > 0) {
+                unsigned* seed;
+                TRY(c->sub[i]->ensure(c->sub[i]->lseed, inst[i].n, &seed));
+                ThrPlan pre = x.pl;
+                pre.a.m = seeds * BI_TC;
+                pre.a.lfin_key = seed;
+                TcInstance* t = &c->batch_host[count + seeded++];
+                TRY(threshold_descriptor(x.ps, pre, x.it, t));
+                t->unit_begin = seed_units;
+                seed_units += (inst[i].n + BU - 1) / BU;
+                x.pl.a.lfin_seed = seed;
+            }
+            TRY(threshold_descriptor(x.ps, x.pl, x.it, &c->batch_host[j]));
             c->batch_host[j].unit_begin = units;
             units += (inst[i].n + BU - 1) / BU;
         }
-        CUDA_TRY(cudaMemcpyAsync(dev, c->batch_host, (size_t)count * sizeof(TcInstance), cudaMemcpyHostToDevice, s));
+        CUDA_TRY(cudaMemcpyAsync(dev, c->batch_host, (size_t)(count + seeded) * sizeof(TcInstance),
+                                 cudaMemcpyHostToDevice, s));
+        if (seeded > 0)
+            launch_threshold_tc(dev + count, seeded, seed_units, kheap, max_dp, w[0].ps.fp8, nseg, true, c->num_sms, s);
         launch_threshold_tc(dev, count, units, kheap, max_dp, w[0].ps.fp8, nseg, false, c->num_sms, s);
         return batch_enqueue_tc(c, inst, count, w, max_dp, s);
     } else {
