@@ -93,6 +93,11 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 // 16-bit bucket of a float, monotone non-decreasing in x.
 __host__ __device__ __forceinline__ uint32_t bucket16(float x) { return float_key(x) >> 16; }
 
+// The largest float of the bucket of x >= 0.  Items are ordered by bucket only, so a later tile can
+// hold a larger norm than an earlier one's maximum, but none above the end of its bucket (NaN for
+// x = inf: a comparison with it is false).
+__device__ __forceinline__ float bucket_end(float x) { return __uint_as_float(__float_as_uint(x) | 0xffffu); }
+
 // Monotone map double -> uint64 for the exact scores; callers add +0.0 first so
 // that -0.0 and +0.0 share one key.
 __device__ __forceinline__ unsigned long long double_key(double s) {

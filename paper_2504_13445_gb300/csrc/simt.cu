@@ -144,10 +144,11 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_threshold_simt(ThresholdArg
                     sel_chunk(v, active, (int)(it * BI_SIMT + c0), a.m, E, s, mycand, a.cap, heap, t,
                               a.k, a.st);
                 }
-                // Algorithm 1's stop by Cauchy-Schwarz: items come in descending norm order, so
-                // once ||u|| max||p|| of the next tile (rounded up) is below a lower bound of
-                // tau_u, no later item can reach tau_u or tie it.
-                need_next = active && it + 1 < item_tiles && !(__fmul_ru(un, a.tmax[it + 1]) < sel_bound(s));
+                // Algorithm 1's stop by Cauchy-Schwarz: items come in descending order of their
+                // norms' buckets, so once ||u|| times the end of the next tile's bucket (rounded
+                // up) is below a lower bound of tau_u, no later item can reach tau_u or tie it.
+                need_next = active && it + 1 < item_tiles &&
+                            !(__fmul_ru(un, bucket_end(a.tmax[it + 1])) < sel_bound(s));
             }
             ++tiles_done;
             if (!__syncthreads_or(need_next)) break;

@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                     tdl_next = tdel[it + 2];
                 }
                 const bool ahead_ok = it + STOP_AHEAD < item_tiles;
-                const float ahead = ahead_ok ? tmax[it + STOP_AHEAD] : 0.f;
+                const float ahead = ahead_ok ? bucket_end(tmax[it + STOP_AHEAD]) : 0.f;
                 if (!mbar_wait(&B->tfull[b], use & 1u, abort, st)) {
                     ok = false;
                     break;
@@ -652,9 +652,10 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                     sel_merge(s, mycand, heap, r, k, active);
                     since = 0;
                 }
-                // Algorithm 1's stop by Cauchy-Schwarz: items arrive in descending norm order,
-                // so once ||u|| max||p|| of a tile (rounded up) is below a lower bound of tau_u,
-                // no item of that tile or any later one can reach tau_u or tie it.  A warp tests
+                // Algorithm 1's stop by Cauchy-Schwarz: items arrive in descending order of their
+                // norms' buckets, so once ||u|| times the end of a tile's bucket (rounded up) is
+                // below a lower bound of tau_u, no item of that tile or any later one can reach
+                // tau_u or tie it.  A warp tests
                 // the tile STOP_AHEAD tiles on (more than the ring and the accumulators hold, so the
                 // producer has not loaded it yet) and publishes its index once none of its users
                 // needs it.  (Searching for the first such tile after every own tile took 450 of
