@@ -887,8 +887,10 @@ int64_t grown_band_cap(const rkm_ctx* c) {
 // Initial capacities of a call: the option (or a default sized from n and k), or the
 // capacity a previous call on this context grew to, whichever is larger.
 void init_caps(rkm_ctx* c, int64_t n, int k) {
-    // FP8's guard band is about eight times BF16's, so its lists start larger.
-    const int dflt = c->opts.precision == RKM_FP8 ? 8 * k + 256 : 2 * k + 96;
+    // FP8's guard band is about eight times BF16's, so its lists start larger: at 100K x 50K, k = 10,
+    // some users need more than 352 slots (8 k + 256) per segment, and the overflow, a compaction
+    // per hit and a second pass made a context's first call 40 ms instead of 6.
+    const int dflt = c->opts.precision == RKM_FP8 ? 16 * k + 512 : 2 * k + 96;
     int cap = c->opts.cand_capacity > 0 ? c->opts.cand_capacity : (int)round_up(dflt, 32);
     cap = (int)round_up(cap, 32);
     if (c->cand_k == k) cap = std::max(cap, c->cand_cap);
