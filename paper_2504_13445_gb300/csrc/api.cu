@@ -555,11 +555,11 @@ struct ThrPlan {
     int nseg, cap;
 };
 
-// Candidate segments per user of a threshold launch with the largest k `kheap` (one per
-// epilogue warpgroup of the tensor-core kernel; one on the FP32 path).  want_groups: the
-// context's epilogue_groups option (0 = auto).
-int threshold_segments(const PathShape& ps, int kheap, int want_groups) {
-    return ps.tc ? threshold_groups(kheap, ps.dp, ps.fp8, want_groups) : 1;
+// Candidate segments per user of a threshold launch of n users and m items with the largest k
+// `kheap` (one per epilogue warpgroup of the tensor-core kernel, from the context's epilogue_groups
+// option; two per part of the items on the FP32 path).
+int threshold_segments(const rkm_ctx* c, const PathShape& ps, int kheap, int64_t n, int64_t m) {
+    return ps.tc ? threshold_groups(kheap, ps.dp, ps.fp8, c->opts.epilogue_groups) : simt_segments(n, m, c->num_sms);
 }
 
 // nseg: candidate segments of the launch this problem joins (0 = a launch of its own).
@@ -571,7 +571,7 @@ rkm_status threshold_prepare(rkm_ctx* c, const PathShape& ps, const float* U, in
         TRY(pack(c, ps, U, n, ldu, d, nullptr, pl->n_pad, c->u_pack, &pl->apack, s, up.e));
     }
     pl->cap = c->cand_cap;
-    pl->nseg = nseg > 0 ? nseg : threshold_segments(ps, k, c->opts.epilogue_groups);
+    pl->nseg = nseg > 0 ? nseg : threshold_segments(c, ps, k, n, it.m);
     TRY(c->ensure(c->cand, n * (int64_t)pl->nseg * pl->cap, &pl->cand));
     TRY(c->ensure(c->cand_cnt, n * (int64_t)pl->nseg, &pl->cand_cnt));
     TRY(c->ensure(c->lfin, n, &pl->lfin));
@@ -725,14 +725,15 @@ rkm_status thresholds_core(rkm_ctx* c, const PathShape& ps, const float* U, int6
                            const float* P, int64_t ldp, int d, int k, const RowPrep& up, const ItemSide& it,
                            double* tau, int* tid, int* topk, cudaStream_t s) {
     for (int attempt = 0;; ++attempt) {
-        const int64_t per_user = (int64_t)threshold_segments(ps, k, c->opts.epilogue_groups) * c->cand_cap * (int64_t)sizeof(Cand);
+        const int nseg = threshold_segments(c, ps, k, n, it.m);
+        const int64_t per_user = (int64_t)nseg * c->cand_cap * (int64_t)sizeof(Cand);
         const int64_t slice = std::min<int64_t>(n, std::max<int64_t>(BU, candidate_budget(c) / per_user / BU * BU));
         bool overflow = false;
         for (int64_t u0 = 0; u0 < n && !overflow; u0 += slice) {
             const int64_t un = std::min<int64_t>(slice, n - u0);
             const RowPrep us = row_slice(up, u0, d);
             ThrPlan pl;
-            TRY(threshold_prepare(c, ps, U + u0 * ldu, un, ldu, d, k, us, it, &pl, s));
+            TRY(threshold_prepare(c, ps, U + u0 * ldu, un, ldu, d, k, us, it, &pl, s, nseg));
             const int64_t seeds = ps.tc && c->opts.seed_order && slice >= n ? seed_tiles(ps, it.tiles, k) : 0;
             if (seeds > 0) TRY(threshold_seed_order(c, ps, U, n, ldu, d, up, it, &pl, seeds, s));
             TRY(threshold_launch_one(c, ps, pl, it, s));
@@ -1774,7 +1775,7 @@ rkm_status batch_enqueue(rkm_ctx* c, const rkm_instance* inst, int count, cudaSt
         max_dp = std::max(max_dp, path_shape(c->opts.precision, inst[i].d).dp);
     }
     const PathShape ps0 = path_shape(c->opts.precision, inst[0].d);
-    const int nseg = ps0.tc ? threshold_groups(kheap, max_dp, ps0.fp8, c->opts.epilogue_groups) : 1;
+    const int nseg = ps0.tc ? threshold_groups(kheap, max_dp, ps0.fp8, c->opts.epilogue_groups) : 0;
     TRY(fork_sides(c, s));
     const auto prepare = [&](int i) -> rkm_status {
         rkm_ctx* sc = c->sub[i];

@@ -58,7 +58,6 @@ struct SelState {
     int cnt;     // candidates stored
     unsigned long long* pub;  // where this group publishes its bound for the other (null: none)
     unsigned tag;             // user tile the published bound belongs to
-    int defer;   // 1: hits only record candidates; sel_merge_tile admits them at the tile's end
     int mark;    // first candidate not yet offered to the heap (-1 after a compaction)
     float Em;    // largest error bound of the tiles since
 };
@@ -100,39 +99,22 @@ __device__ __forceinline__ void heapify(float* heap, int t, int k) {
     }
 }
 
-// Record a value that reached the threshold: store it as a candidate (with its upper bound),
-// and admit its lower bound into the heap when it raises the best bound known here.  Any k
-// lower bounds held in the heap make its root a valid lower bound of tau_u, so skipping an
-// admission is sound; while the heap fills, admission is an append, and the heap is built
-// once when it holds k values.
+// Record a value that reached the threshold: store it as a candidate (with its upper bound).  Its
+// lower bound enters the heap later (sel_merge): any k lower bounds held in the heap make its root
+// a valid lower bound of tau_u, so delaying or skipping an admission is sound.
 __device__ __forceinline__ void sel_insert(float v, int pos, float E, SelState& s, Cand* mycand, int cap,
-                                           float* heap, int t, int k, DevStatus* st) {
-    const float ub = __fadd_ru(v, E);
-    const float lb = __fsub_rd(v, E);
+                                           DevStatus* st) {
     if (s.cnt >= cap) {
         s.cnt = compact_candidates(mycand, s.cnt, sel_bound(s));
         s.mark = -1;
     }
     if (s.cnt < cap) {
         Cand c;
-        c.ub = ub;
+        c.ub = __fadd_ru(v, E);
         c.pos = pos;
         mycand[s.cnt++] = c;
     } else {
         st->cand_overflow = 1u;
-    }
-    if (s.defer) return;
-    if (lb > sel_bound(s)) {
-        if (s.hn < k) {
-            heap[s.hn * BU + t] = lb;
-            if (++s.hn < k) return;
-            heapify(heap, t, k);
-        } else {
-            heap_replace_root(heap, t, k, lb);
-        }
-        s.L = heap[t];
-        if (s.pub) publish_bound(s.pub, s.tag, fmaxf(s.L, s.Lw));
-        s.thr = __fsub_rd(sel_bound(s), E);
     }
 }
 
@@ -143,6 +125,11 @@ __device__ __forceinline__ float cand_lower(float ub, float E) {
     const float d = __fadd_ru(__fmul_ru(fabsf(ub), 0x1p-23f), 0x1p-149f);
     return __fsub_rd(__fsub_rd(__fsub_rd(ub, E), E), d);
 }
+
+// A selector offers its candidates to the heap after MERGE_TILES of its tiles, or once some row of
+// the warp has MERGE_HITS new ones.
+constexpr int MERGE_TILES = 8;
+constexpr int MERGE_HITS = 2;
 
 // Deferred admissions: the lower bounds of the candidates recorded since the last call enter the
 // heap with every lane of the warp stepping through its own list together (the heap is built at
@@ -236,13 +223,12 @@ __device__ __forceinline__ unsigned hit_mask(const float (&v)[32], const float (
 // lane reaches its threshold are compared element by element, and the hits are inserted one
 // by one through a single call site.  `active` masks lanes without a valid user.
 __device__ __forceinline__ void sel_chunk(const float (&v)[32], bool active, int pos0, int64_t m,
-                                          float E, SelState& s, Cand* mycand, int cap, float* heap,
-                                          int t, int k, DevStatus* st) {
+                                          float E, SelState& s, Cand* mycand, int cap, DevStatus* st) {
     float g[4];
     group_max8(v, g);
     const float mx = fmax3f(g[0], g[1], fmaxf(g[2], g[3]));
     if (!__any_sync(0xffffffffu, active && mx >= s.thr)) return;
-    if (s.defer && pos0 + 32 <= m && !__any_sync(0xffffffffu, active && s.cnt + 32 > cap)) {
+    if (pos0 + 32 <= m && !__any_sync(0xffffffffu, active && s.cnt + 32 > cap)) {
         // Room for the whole chunk and no column past the items: the columns of each 8-column
         // group with a hit are compared and stored in place, without a branch per hit.
         Cand* p = mycand + s.cnt;
@@ -271,7 +257,7 @@ __device__ __forceinline__ void sel_chunk(const float (&v)[32], bool active, int
         mask &= mask - 1u;
         const float x = select32(v, c);
         // s.thr only grows, so skipping values now below it is still sound.
-        if (x >= s.thr && pos0 + c < m) sel_insert(x, pos0 + c, E, s, mycand, cap, heap, t, k, st);
+        if (x >= s.thr && pos0 + c < m) sel_insert(x, pos0 + c, E, s, mycand, cap, st);
     }
 }
 

@@ -113,6 +113,8 @@ struct ThresholdArgs {
     const int* uperm;
     const unsigned* lfin_seed;
 };
+// Candidate segments per user of an FP32 threshold launch: two for each part of the item tiles.
+int simt_segments(int64_t n, int64_t m, int num_sms);
 void launch_threshold_simt(const ThresholdArgs& a, cudaStream_t s);
 
 // One problem of the tensor-core threshold pass: its TMA descriptors (users, items), its

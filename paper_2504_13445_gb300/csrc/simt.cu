@@ -5,6 +5,8 @@
 // memory and handed row by row to the per-user epilogues of epilogue.cuh.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "count_units.cuh"
 #include "epilogue.cuh"
@@ -19,11 +21,20 @@ constexpr int ASTR = 132;       // row stride (floats) of the transposed operand
 constexpr int CSTR = 132;       // row stride of the staged score tile
 constexpr int SIMT_THREADS = 256;
 
-struct SimtSmem {
-    float As[KC * ASTR];        // users chunk, [k][user]
-    float Bs[KC * ASTR];        // items chunk, [k][item]
+// The staged scores take the place of the operand chunks, which the product has finished with, so
+// that two CTAs fit an SM: one's product then runs beside the other's epilogue (counting phase at
+// 20,000 users x 5,000 items, d = 64: 416 -> 360 us).
+union SimtSmem {
+    struct {
+        float As[KC * ASTR];    // users chunk, [k][user]
+        float Bs[KC * ASTR];    // items chunk, [k][item]
+    };
     float Cs[BU * CSTR];        // scores, [user][item]
 };
+constexpr int SIMT_CTAS = 2;             // per SM
+constexpr int SIMT_PARTS = 4;            // most parts of the item tiles (simt_segments)
+constexpr int SIMT_HALF = BI_SIMT / 2;   // columns of a tile that one thread of the epilogue reads
+static_assert(SIMT_THREADS == 2 * BU && BU == 128, "two threads of the epilogue per user");
 
 // Load a 128-row x 32-k chunk of a packed operand (row stride dp) transposed into S[k][row].
 __device__ __forceinline__ void load_chunk_t(const float* __restrict__ X, int64_t row0, int dp, int k0,
@@ -93,80 +104,95 @@ __device__ __forceinline__ void load_row_chunk(const SimtSmem& sm, int row, int 
     }
 }
 
-// K2: persistent over user tiles; every CTA scans all item tiles for its users.
-__global__ void __launch_bounds__(SIMT_THREADS, 1) k_threshold_simt(ThresholdArgs a) {
+// K2: one CTA per user tile and part p of the item tiles (p, p + parts, ...), part after part.  A
+// thread of the epilogue selects among half the columns of its user's row, into a list segment and
+// a heap of its own; the 2 * parts threads of a user share their bounds through lfin_key.
+// Bound by FP32 issue and by the epilogue of half a CTA's warps, which the other half and the
+// other CTA of the SM now fill: 20,000 users x 5,000 items, d = 64, k = 25, where 157 user tiles took
+// two rounds of one CTA per SM: 862 -> 502 us (two CTAs per SM alone: 735).
+__global__ void __launch_bounds__(SIMT_THREADS, SIMT_CTAS) k_threshold_simt(ThresholdArgs a, int parts) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SimtSmem& sm = *reinterpret_cast<SimtSmem*>(smem_raw);
-    float* heap = reinterpret_cast<float*>(smem_raw + sizeof(SimtSmem));  // [k][BU]
     const float* A = static_cast<const float*>(a.A);
     const float* B = static_cast<const float*>(a.B);
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, r = t & (BU - 1), half = t >> 7;
+    float* heap = reinterpret_cast<float*>(smem_raw + sizeof(SimtSmem)) + (size_t)half * a.k * BU;  // [2][k][BU]
     const int64_t user_tiles = (a.n + BU - 1) / BU;
     const int64_t item_tiles = (a.m + BI_SIMT - 1) / BI_SIMT;
-    for (int64_t ut = blockIdx.x; ut < user_tiles; ut += gridDim.x) {
-        const int64_t u = ut * BU + t;
-        const bool owner = t < BU;
-        const bool active = owner && u < a.n;
-        SelState s;
-        s.L = -INFINITY;
-        s.hn = 0;
-        s.Lw = -INFINITY;
-        s.Lx = -INFINITY;
-        s.thr = -INFINITY;
-        s.cnt = 0;
-        s.pub = nullptr;
-        s.tag = 0u;
-        s.defer = 0;
-        s.mark = 0;
-        s.Em = 0.f;
-        float un = 0.f, unh = 0.f, ud = 0.f;
-        Cand* mycand = nullptr;
-        if (owner) {
-            for (int j = 0; j < a.k; ++j) heap[j * BU + t] = -INFINITY;
-            if (active) {
-                un = a.unrm[u];
-                unh = a.unhat[u];
-                ud = a.udel[u];
-                mycand = a.cand + u * (int64_t)a.nseg * a.cap;
-            }
+    const int64_t ut = blockIdx.x % user_tiles;
+    const int part = (int)(blockIdx.x / user_tiles);
+    const int64_t u = ut * BU + r;
+    const bool active = u < a.n;
+    const int seg = part * 2 + half;
+    SelState s;
+    s.L = -INFINITY;
+    s.hn = 0;
+    s.Lw = -INFINITY;
+    s.Lx = -INFINITY;
+    s.thr = -INFINITY;
+    s.cnt = 0;
+    s.pub = nullptr;
+    s.tag = 0u;
+    s.mark = 0;
+    s.Em = 0.f;
+    for (int j = 0; j < a.k; ++j) heap[j * BU + r] = -INFINITY;
+    const float un = active ? a.unrm[u] : 0.f;
+    const float unh = active ? a.unhat[u] : 0.f;
+    const float ud = active ? a.udel[u] : 0.f;
+    Cand* mycand = a.cand + ((active ? u : 0) * a.nseg + seg) * (int64_t)a.cap;
+    bool warm = false;
+    int since = 0;               // tiles since candidates were offered to the heap
+    float published = -INFINITY;
+    int64_t items = 0;
+    for (int64_t it = part; it < item_tiles; it += parts) {
+        // Any bound the other threads of this user have published bounds tau_u from below.
+        const unsigned lk = active ? __ldcg(&a.lfin_key[u]) : 0u;
+        simt_tile(A, ut * BU, B, it * BI_SIMT, a.dp, sm);
+        s.Lx = key_float(lk);
+        const float E = err_bound(a.cacc, a.eabs, un, unh, ud, a.thmax[it], a.tdel[it]);
+        const int pos0 = (int)(it * BI_SIMT) + half * SIMT_HALF;
+        if (!warm) {
+            // A lower bound before any candidate is recorded (see warm_bound): the k-th largest of
+            // 32 maxima of 2 columns, -inf for k > 32.
+            auto load = [&](int c0, float (&v)[32]) { load_row_chunk(sm, r, half * SIMT_HALF + c0, v); };
+            const float lw = warm_bound<32, SIMT_HALF>(load, pos0, a.m, a.k, E);
+            s.Lw = active ? lw : -INFINITY;
+            warm = true;
         }
-        int64_t tiles_done = 0;
-        for (int64_t it = 0; it < item_tiles; ++it) {
-            simt_tile(A, ut * BU, B, it * BI_SIMT, a.dp, sm);
-            bool need_next = false;
-            if (owner) {
-                const float E = err_bound(a.cacc, a.eabs, un, unh, ud, a.thmax[it], a.tdel[it]);
-                s.thr = __fsub_rd(sel_bound(s), E);
+        s.thr = __fsub_rd(sel_bound(s), E);
 #pragma unroll 1
-                for (int c0 = 0; c0 < BI_SIMT; c0 += 32) {
-                    float v[32];
-                    load_row_chunk(sm, t, c0, v);
-                    sel_chunk(v, active, (int)(it * BI_SIMT + c0), a.m, E, s, mycand, a.cap, heap, t,
-                              a.k, a.st);
-                }
-                // Algorithm 1's stop by Cauchy-Schwarz: items come in descending order of their
-                // norms' buckets, so once ||u|| times the end of the next tile's bucket (rounded
-                // up) is below a lower bound of tau_u, no later item can reach tau_u or tie it.
-                need_next = active && it + 1 < item_tiles &&
-                            !(__fmul_ru(un, bucket_end(a.tmax[it + 1])) < sel_bound(s));
-            }
-            ++tiles_done;
-            if (!__syncthreads_or(need_next)) break;
+        for (int c0 = 0; c0 < SIMT_HALF; c0 += 32) {
+            float v[32];
+            load_row_chunk(sm, r, half * SIMT_HALF + c0, v);
+            sel_chunk(v, active, pos0 + c0, a.m, E, s, mycand, a.cap, a.st);
         }
-        if (t == 0) {
-            const int64_t rows = (a.n - ut * BU < BU) ? a.n - ut * BU : BU;
-            const int64_t items = (tiles_done * BI_SIMT < a.m) ? tiles_done * BI_SIMT : a.m;
-            atomicAdd(&a.st->thr_pairs, (unsigned long long)(rows * items));
+        s.Em = fmaxf(s.Em, E);
+        if (++since == MERGE_TILES || __any_sync(0xffffffffu, active && s.mark >= 0 && s.cnt - s.mark >= MERGE_HITS)) {
+            sel_merge(s, mycand, heap, r, a.k, active);
+            since = 0;
         }
-        if (active) {
-            atomicMax(&a.lfin_key[u], float_key(fmaxf(s.L, s.Lw)));
-            a.cand_cnt[u * a.nseg] = s.cnt;
+        const float own = fmaxf(s.L, s.Lw);
+        if (active && own > published) {
+            published = own;
+            atomicMax(&a.lfin_key[u], float_key(own));
         }
+        items += a.m - it * BI_SIMT < BI_SIMT ? a.m - it * BI_SIMT : BI_SIMT;
+        // Algorithm 1's stop by Cauchy-Schwarz: items come in descending order of their norms'
+        // buckets, so once ||u|| times the end of the next tile's bucket (rounded up) is below a
+        // lower bound of tau_u, no later item can reach tau_u or tie it.
+        const bool need_next =
+            active && it + parts < item_tiles && !(__fmul_ru(un, bucket_end(a.tmax[it + parts])) < sel_bound(s));
+        if (!__syncthreads_or(need_next)) break;
     }
+    if (t == 0) {
+        const int64_t rows = (a.n - ut * BU < BU) ? a.n - ut * BU : BU;
+        atomicAdd(&a.st->thr_pairs, (unsigned long long)(rows * items));
+    }
+    if (active) a.cand_cnt[u * a.nseg + seg] = s.cnt;
 }
 
 // K5: persistent over work units (item tile, group of user tiles) taken from a ticket.
-__global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
+__global__ void __launch_bounds__(SIMT_THREADS, SIMT_CTAS) k_count_simt(CountArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SimtSmem& sm = *reinterpret_cast<SimtSmem*>(smem_raw);
     int* cnt_s = reinterpret_cast<int*>(smem_raw + sizeof(SimtSmem));  // [BI_SIMT]
@@ -182,7 +208,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
         const unsigned w = s_unit;
         __syncthreads();
         if (w >= total) {
-            if (t < BU) band_flush(stage, a.band, a.band_cap, a.st);
+            band_flush(stage, a.band, a.band_cap, a.st);
             break;
         }
         int T;
@@ -194,27 +220,26 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
         const int pos0 = T * BI_SIMT;
         for (int64_t ut = ut0; ut < ut1; ++ut) {
             simt_tile(A, ut * BU, B, (int64_t)T * BI_SIMT, a.dp, sm);
-            if (t < BU) {
-                const int64_t us = ut * BU + t;
-                const bool active = us < a.n;
-                float hi_t = 0.f, lo_t = 0.f;
-                int u_orig = 0;
-                if (active) {
-                    const UserMeta um = a.meta[us];
-                    const float E = err_bound(a.cacc, a.eabs, um.un, um.unh, um.ud, pnh, pd);
-                    hi_t = __fadd_ru(um.tau_hi, E);
-                    lo_t = __fsub_rd(um.tau_lo, E);
-                    u_orig = um.uorig;
-                }
-#pragma unroll 1
-                for (int c0 = 0; c0 < BI_SIMT; c0 += 32) {
-                    float v[32];
-                    load_row_chunk(sm, t, c0, v);
-                    count_chunk(v, active, c0, pos0 + c0, a.m, hi_t, lo_t, cnt_s, u_orig, stage, a.band,
-                                a.band_cap, a.st);
-                }
-                if (stage.n > BAND_STAGE / 2) band_flush(stage, a.band, a.band_cap, a.st);
+            const int r = t & (BU - 1), h0 = (t >> 7) * SIMT_HALF;
+            const int64_t us = ut * BU + r;
+            const bool active = us < a.n;
+            float hi_t = 0.f, lo_t = 0.f;
+            int u_orig = 0;
+            if (active) {
+                const UserMeta um = a.meta[us];
+                const float E = err_bound(a.cacc, a.eabs, um.un, um.unh, um.ud, pnh, pd);
+                hi_t = __fadd_ru(um.tau_hi, E);
+                lo_t = __fsub_rd(um.tau_lo, E);
+                u_orig = um.uorig;
             }
+#pragma unroll 1
+            for (int c0 = h0; c0 < h0 + SIMT_HALF; c0 += 32) {
+                float v[32];
+                load_row_chunk(sm, r, c0, v);
+                count_chunk(v, active, c0, pos0 + c0, a.m, hi_t, lo_t, cnt_s, u_orig, stage, a.band, a.band_cap,
+                            a.st);
+            }
+            if (stage.n > BAND_STAGE / 2) band_flush(stage, a.band, a.band_cap, a.st);
             __syncthreads();
         }
         if (t == 0 && ut1 > ut0) {
@@ -228,21 +253,32 @@ __global__ void __launch_bounds__(SIMT_THREADS, 1) k_count_simt(CountArgs a) {
 
 }  // namespace
 
+// Parts of the item tiles: as many as give each CTA slot of the SMs about four units, at most
+// SIMT_PARTS.  Each part selects on its own, so more parts record more candidates: at 20,000 users x
+// 5,000 items, k = 25, threshold and exact phase take 735 + 35 us with one part (and one thread per
+// row), 608 + 68 with two, 502 + 102 with four, 471 + 248 with eight.
+int simt_segments(int64_t n, int64_t m, int num_sms) {
+    const int64_t user_tiles = (n + BU - 1) / BU, item_tiles = (m + BI_SIMT - 1) / BI_SIMT;
+    const int64_t want = ((int64_t)4 * SIMT_CTAS * num_sms + user_tiles - 1) / std::max<int64_t>(user_tiles, 1);
+    return 2 * (int)std::max<int64_t>(1, std::min<int64_t>({want, SIMT_PARTS, item_tiles}));
+}
+
 void launch_threshold_simt(const ThresholdArgs& a, cudaStream_t s) {
-    const size_t smem = sizeof(SimtSmem) + (size_t)KMAX * BU * sizeof(float);
-    cudaFuncSetAttribute(k_threshold_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int64_t user_tiles = (a.n + BU - 1) / BU;
-    int grid = (int)(user_tiles < a.num_sms ? user_tiles : a.num_sms);
-    if (grid < 1) return;
+    const size_t smem = sizeof(SimtSmem) + (size_t)2 * a.k * BU * sizeof(float);
+    cudaFuncSetAttribute(k_threshold_simt, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sizeof(SimtSmem) + (size_t)2 * KMAX * BU * sizeof(float)));
+    const int parts = a.nseg / 2;
+    const int64_t units = (a.n + BU - 1) / BU * parts;
+    if (units < 1) return;
     note_launch();
-    k_threshold_simt<<<grid, SIMT_THREADS, smem, s>>>(a);
+    k_threshold_simt<<<(unsigned)units, SIMT_THREADS, smem, s>>>(a, parts);
 }
 
 void launch_count_simt(const CountArgs& a, cudaStream_t s) {
-    const size_t smem = sizeof(SimtSmem) + BI_SIMT * sizeof(int) + (BU / 32) * BAND_STAGE * sizeof(int2);
+    const size_t smem = sizeof(SimtSmem) + BI_SIMT * sizeof(int) + (SIMT_THREADS / 32) * BAND_STAGE * sizeof(int2);
     cudaFuncSetAttribute(k_count_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     note_launch();
-    k_count_simt<<<a.num_sms, SIMT_THREADS, smem, s>>>(a);
+    k_count_simt<<<a.num_sms * SIMT_CTAS, SIMT_THREADS, smem, s>>>(a);
 }
 
 }  // namespace rkm

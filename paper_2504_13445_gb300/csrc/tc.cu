@@ -38,8 +38,6 @@ namespace {
 constexpr int tc_threads(int ng) { return 64 + 128 * ng; }
 constexpr int MAX_SLOTS = 4;
 constexpr int STOP_AHEAD = 8;   // tiles between the stop's test and the tile it tests
-constexpr int MERGE_TILES = 8;  // own tiles, or
-constexpr int MERGE_HITS = 2;   // candidates of one row, between admissions to the heap
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t KB_BYTES_U = 128 * 128;  // one K-block (128 bytes: 64 BF16 / 128 FP8) of 128 user rows
 constexpr uint32_t KB_BYTES_I = 256 * 128;  // one K-block of 256 item rows
@@ -528,7 +526,6 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
             s.cnt = 0;
             s.pub = &Lpub[g * BU + r];
             s.tag = (unsigned)w;
-            s.defer = 1;
             s.mark = 0;
             s.Em = 0.f;
             bool warm = a.lfin_seed != nullptr;  // warm start done for this unit (or seeded)
@@ -635,8 +632,8 @@ __global__ void __launch_bounds__(tc_threads(NG), 1)
                             scale_values(va, f);
                             scale_values(vb, f);
                         }
-                        sel_chunk(va, active, it * BI_TC + cg + c0, m, E, s, mycand, cap, heap, r, k, st);
-                        sel_chunk(vb, active, it * BI_TC + cg + c0 + 32, m, E, s, mycand, cap, heap, r, k, st);
+                        sel_chunk(va, active, it * BI_TC + cg + c0, m, E, s, mycand, cap, st);
+                        sel_chunk(vb, active, it * BI_TC + cg + c0 + 32, m, E, s, mycand, cap, st);
                     }
                 }
                 tc_fence_before();
