@@ -445,13 +445,14 @@ struct RowPrep {
     float* nrm;   // ||x|| rounded up
     float* nhat;  // ||x^|| rounded up (x^ = operand of the product kernels)
     float* del;   // ||x^ - x|| rounded up
+    void* pack = nullptr;  // BF16 operand rows in this order, when the preparation made them
 };
 
 // Users get the norms of their product operand here; items on the FP8 path get them from
 // their pack, whose scale is per item tile (items = true).
 rkm_status prep_rows(rkm_ctx* c, const PathShape& ps, const float* X, int64_t rows, int64_t ld, int d, Buf& be,
                      Buf& bq, Buf& bn2, Buf& bnrm, Buf& bnhat, Buf& bdel, RowPrep* out, cudaStream_t s,
-                     bool items = false) {
+                     bool items = false, Buf* bpack = nullptr) {
     const int dq = (int)round_up(d, 8);
     TRY(c->ensure(be, rows, &out->e));
     TRY(c->ensure(bq, rows * dq, &out->q));
@@ -460,7 +461,12 @@ rkm_status prep_rows(rkm_ctx* c, const PathShape& ps, const float* X, int64_t ro
     TRY(c->ensure(bnhat, rows, &out->nhat));
     TRY(c->ensure(bdel, rows, &out->del));
     const int operand = !ps.tc ? OPERAND_F32 : !ps.fp8 ? OPERAND_BF16 : items ? OPERAND_F32 : OPERAND_FP8_ROW;
-    launch_prep_rows(X, rows, ld, d, out->e, out->q, dq, out->n2, out->nrm, out->nhat, out->del, operand, c->st, s);
+    __nv_bfloat16* pack = nullptr;
+    const int64_t rows_pad = round_up(std::max<int64_t>(rows, 1), BU);
+    if (bpack && operand == OPERAND_BF16) TRY(c->ensure(*bpack, rows_pad * ps.dp, &pack));
+    out->pack = pack;
+    launch_prep_rows(X, rows, ld, d, out->e, out->q, dq, out->n2, out->nrm, out->nhat, out->del, operand, c->st, s,
+                     pack, rows_pad, ps.dp);
     return RKM_OK;
 }
 
@@ -566,7 +572,9 @@ int threshold_segments(const rkm_ctx* c, const PathShape& ps, int kheap, int64_t
 rkm_status threshold_prepare(rkm_ctx* c, const PathShape& ps, const float* U, int64_t n, int64_t ldu, int d, int k,
                              const RowPrep& up, const ItemSide& it, ThrPlan* pl, cudaStream_t s, int nseg = 0) {
     pl->n_pad = round_up(std::max<int64_t>(n, 1), BU);
-    {
+    if (up.pack) {
+        pl->apack = up.pack;
+    } else {
         Phase ph(c, s, RKM_PHASE_PREP);
         TRY(pack(c, ps, U, n, ldu, d, nullptr, pl->n_pad, c->u_pack, &pl->apack, s, up.e));
     }
@@ -713,9 +721,10 @@ int64_t candidate_budget(const rkm_ctx* c) {
 }
 
 // Rows [u0, u0 + rows) of a prepared side.
-RowPrep row_slice(const RowPrep& r, int64_t u0, int d) {
+RowPrep row_slice(const RowPrep& r, int64_t u0, int d, int dp) {
     const int64_t dq = round_up(d, 8);
-    return RowPrep{r.e + u0, r.q + u0 * dq, r.n2 + u0, r.nrm + u0, r.nhat + u0, r.del + u0};
+    return RowPrep{r.e + u0, r.q + u0 * dq, r.n2 + u0, r.nrm + u0, r.nhat + u0, r.del + u0,
+                   r.pack ? static_cast<__nv_bfloat16*>(r.pack) + u0 * dp : nullptr};
 }
 
 // Thresholds of every user, in slices of users small enough that their candidate lists fit
@@ -731,7 +740,8 @@ rkm_status thresholds_core(rkm_ctx* c, const PathShape& ps, const float* U, int6
         bool overflow = false;
         for (int64_t u0 = 0; u0 < n && !overflow; u0 += slice) {
             const int64_t un = std::min<int64_t>(slice, n - u0);
-            const RowPrep us = row_slice(up, u0, d);
+            RowPrep us = row_slice(up, u0, d, ps.dp);
+            if (attempt > 0) us.pack = nullptr;  // the seed order has packed over it
             ThrPlan pl;
             TRY(threshold_prepare(c, ps, U + u0 * ldu, un, ldu, d, k, us, it, &pl, s, nseg));
             const int64_t seeds = ps.tc && c->opts.seed_order && slice >= n ? seed_tiles(ps, it.tiles, k) : 0;
@@ -1077,7 +1087,8 @@ rkm_status rkm_thresholds(rkm_ctx* c, const float* U, int64_t n, int64_t ldu, co
     ItemSide it;
     {
         Phase ph(c, s, RKM_PHASE_PREP);
-        TRY(prep_rows(c, ps, U, n, ldu, d, c->u_e, c->u_q, c->u_n2, c->u_nrm, c->u_nhat, c->u_del, &up, s));
+        TRY(prep_rows(c, ps, U, n, ldu, d, c->u_e, c->u_q, c->u_n2, c->u_nrm, c->u_nhat, c->u_del, &up, s, false,
+                      &c->u_pack));
         TRY(prep_items(c, ps, P, m, ldp, d, catalogue_bufs(c), &it, s));
     }
     TRY(thresholds_core(c, ps, U, n, ldu, P, ldp, d, k, up, it, tau, tid, topk, s));
@@ -1252,7 +1263,8 @@ rkm_status rkm_topn(rkm_ctx* c, const float* U, int64_t n, int64_t ldu, const fl
     ItemSide it;
     {
         Phase ph(c, s, RKM_PHASE_PREP);
-        TRY(prep_rows(c, ps, U, n, ldu, d, c->u_e, c->u_q, c->u_n2, c->u_nrm, c->u_nhat, c->u_del, &up, s));
+        TRY(prep_rows(c, ps, U, n, ldu, d, c->u_e, c->u_q, c->u_n2, c->u_nrm, c->u_nhat, c->u_del, &up, s, false,
+                      &c->u_pack));
         TRY(prep_items(c, ps, P, m, ldp, d, catalogue_bufs(c), &it, s));
     }
     if (c->opts.scores_from_topk) {
@@ -1786,7 +1798,7 @@ rkm_status batch_enqueue(rkm_ctx* c, const rkm_instance* inst, int count, cudaSt
         init_caps(sc, I.n, I.k);
         TRY(begin_call(sc, si));
         TRY(prep_rows(sc, x.ps, I.U, I.n, I.ldu, I.d, sc->u_e, sc->u_q, sc->u_n2, sc->u_nrm, sc->u_nhat, sc->u_del,
-                      &x.up, si));
+                      &x.up, si, false, &sc->u_pack));
         TRY(prep_items(sc, x.ps, I.P, I.m, I.ldp, I.d, catalogue_bufs(sc), &x.it, si));
         TRY(threshold_prepare(sc, x.ps, I.U, I.n, I.ldu, I.d, I.k, x.up, x.it, &x.pl, si, nseg));
         TRY(sc->ensure(sc->tau_tmp, I.n, &x.tau));

@@ -26,11 +26,13 @@ inline void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); 
 // Also ||x^|| and ||x^ - x|| (rounded up) of the operand x^ the product kernels see:
 // OPERAND_F32: x itself; OPERAND_BF16: BF16 round-to-nearest of x; OPERAND_FP8_ROW: x scaled
 // by 2^(8-e), rounded to FP8 e4m3 (nearest even) and scaled back (per-row scale).  Operands
-// with a per-tile scale get their norms from launch_pack_fp8 instead.
+// with a per-tile scale get their norms from launch_pack_fp8 instead.  pack (BF16 operand, may be
+// null): the operand rows in this order, [rows_pad][dp], zero padded.
 enum OperandKind { OPERAND_F32 = 0, OPERAND_BF16 = 1, OPERAND_FP8_ROW = 2 };
 void launch_prep_rows(const float* X, int64_t rows, int64_t ld, int d, int* ex, int16_t* q,
                       int dq, double* norm2, float* nrm_hi, float* nhat_hi, float* del_hi,
-                      int operand, DevStatus* st, cudaStream_t s);
+                      int operand, DevStatus* st, cudaStream_t s, __nv_bfloat16* pack = nullptr,
+                      int64_t rows_pad = 0, int dp = 0);
 
 // FP8 e4m3 operand copy dst[r][c] (rows_pad x dp bytes) of X (row perm[r] if perm != null):
 // row r holds e4m3(x * 2^(8 - e_r)) with e_r = tile_exp[r / tile] when tile_exp != null,
