@@ -817,8 +817,8 @@ rkm_status count_descriptor(const PathShape& ps, int64_t n, const UserOrder& uo,
 
 // User tiles per counting work unit: the context's (32, or the autotuner's), or fewer where that
 // would leave the SMs less than about 8 units each.  2,000 users x 1,000 items made 4 units of 16
-// tiles (81 us on 4 SMs; 64 units of one tile: 22 us), and 32 candidates against a million users
-// 244 units for 152 SMs.  Smaller units than needed reload the resident item tile more often.
+// tiles (counting phase 78 us on 4 SMs; 64 units of one tile: 17 us), and 32 candidates against a
+// million users 244 units for 152 SMs.  Smaller units than needed reload the resident item tile more often.
 int unit_tiles(const rkm_ctx* c, int64_t n, int item_tiles) {
     const int64_t tiles = (n + BU - 1) / BU * item_tiles;
     return (int)std::max<int64_t>(1, std::min<int64_t>(c->count_group, tiles / ((int64_t)c->num_sms * 8)));

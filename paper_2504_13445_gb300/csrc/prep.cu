@@ -34,13 +34,34 @@ inline int grid_for(int64_t work, int per_block, int cap = 1 << 20) {
     return (int)g;
 }
 
+// S * 2^x for an integer 0 < S < 2^53, exactly; the result must be a normal double.
+__device__ __forceinline__ double scaled_integer(unsigned long long S, int x) {
+    const int p = 63 - __clzll((long long)S);
+    return __longlong_as_double(((long long)(p + x + 1023) << 52) | (long long)((S << (52 - p)) & 0xfffffffffffffull));
+}
+
+// The smallest float >= sqrt(S) * 2^x, in integers: FP64 instructions issue at a small fraction of the
+// FP32 rate here, and a square root of one lane holds its whole warp (preparation phase of 2M users x
+// 500K items, d = 128: 2.30 ms with FP64 norms, 1.37 so).  2^22 < S <= 2^32, and the result
+// must be normal.  r <= sqrt(S) within two units in the last place, and a float M 2^(p-23) reaches
+// sqrt(S) iff M^2 >= S 2^(2(23-p)).
+__device__ __forceinline__ float sqrt_up(unsigned long long S, int x) {
+    const float r = __fsqrt_rd(__ull2float_rd(S));
+    int p = (int)(__float_as_uint(r) >> 23) - 127;
+    unsigned long long M = (__float_as_uint(r) & 0x7fffffu) | 0x800000u;
+    const unsigned long long T = S << (2 * (23 - p));
+    while (M * M < T) ++M;
+    p += (int)(M >> 24);  // M = 2^24: the next power of two, whose fraction is 0 as well
+    return __uint_as_float(((unsigned)(p + x + 127) << 23) | ((unsigned)M & 0x7fffffu));
+}
+
 // A segment of lpr lanes per row (lpr a power of two, 32 / lpr rows per warp), eight consecutive
 // elements per lane, read once into registers with 16-byte loads where the rows allow it (vec).
 // The row is on the grid iff every x * 2^(12-e) is an integer of magnitude <= 4096; then
 // ||x||^2 = sum(q^2) * 2^(2e-24) exactly.  With `pack`, also the BF16 operand row (zero beyond d, and
 // zero rows up to rows_pad), which saves a pass over X.  With one element per lane and step, the row
 // read twice and a generic power-of-two scaling per element, 480K rows of d = 200 took 370 us and
-// their pack 160 more; 500 us together so (the preparation phase: 700 -> 636 us).
+// their pack 160 more; 302 us together so.
 template <bool PACK>
 __global__ void __launch_bounds__(256)
     k_prep_rows(const float* __restrict__ X, int64_t rows, int64_t ld, int d, int* __restrict__ ex,
@@ -119,15 +140,23 @@ __global__ void __launch_bounds__(256)
         }
         if (valid && c0 == 0) {
             double n2;
-            if (ok) {
-                n2 = ldexp((double)sum2, 2 * e - 24);  // exact
+            float nrm;
+            if (!ok) {
+                n2 = (double)d2;  // an upper bound
+                nrm = __fsqrt_ru(d2);
+                // Only the first rows off the grid write the flag: with one atomic per row, 480,000 rows
+                // of d = 200 took 500 us, 302 so.
+                if (*reinterpret_cast<volatile unsigned*>(grid_flag) == 0u) atomicOr(grid_flag, 1u);
+            } else if (sum2 > 0 && e >= -120 && e <= 110) {
+                n2 = scaled_integer((unsigned long long)sum2, 2 * e - 24);  // exact
+                nrm = sqrt_up((unsigned long long)sum2, e - 12);
             } else {
-                n2 = (double)d2;                       // an upper bound
-                atomicOr(grid_flag, 1u);
+                n2 = ldexp((double)sum2, 2 * e - 24);
+                nrm = __double2float_ru(__dsqrt_ru(n2));
             }
             ex[row] = e;
             norm2[row] = n2;
-            nrm_hi[row] = ok ? __double2float_ru(__dsqrt_ru(n2)) : __fsqrt_ru(d2);
+            nrm_hi[row] = nrm;
             nhat_hi[row] = __fsqrt_ru(h2);
             del_hi[row] = __fsqrt_ru(e2);
         }
@@ -228,7 +257,7 @@ __global__ void k_tile_exp(const int* __restrict__ ex, const int* __restrict__ p
 // Bucket counts of a block in shared memory, two 16-bit counters to a word (a block counts at most
 // SORT_CHUNK keys at a time).  Keys crowd into a few hundred of the 65,536 buckets (ratios and
 // norms span a few octaves of 128 buckets), so one global atomic per key waited in line: 60 us
-// each for counting and placing 500,000 keys, 8 and 12 us with one atomic per block and bucket.
+// each for counting and placing 500,000 keys, 7 and 8 us with one atomic per block and bucket.
 constexpr int SORT_THREADS = 1024;
 constexpr int SORT_CHUNK = 8192;     // keys a block handles at a time
 constexpr int SORT_SMALL = 16384;    // keys that one block sorts alone
@@ -311,7 +340,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_scatter(const float* __restric
 }
 
 // The whole sort of up to SORT_SMALL keys by one block: one launch instead of a clear and four
-// kernels (about 18 us of launches for 1,000 keys, 9 us so).
+// kernels (about 18 us for 1,000 keys; 5 us so, 9 for 5,000).
 __global__ void __launch_bounds__(SORT_THREADS) k_sort_small(const float* __restrict__ keys, int count, bool desc,
                                                              int* __restrict__ perm, unsigned* __restrict__ cum) {
     extern __shared__ __align__(16) unsigned cnt[];
