@@ -14,11 +14,11 @@
 // decides only between candidates whose FP32 sums are too close, and the FP64 value of tau_u
 // itself is formed for up to 32 users at a time, one per lane.  Against one lane per candidate
 // and a ranking of all of them by shuffles, measured on GB300:
-//   K3, grid      500K users x 100K items, d = 64,  k = 25         1.87 -> 0.84 ms
-//   K3, grid      2M x 500K,               d = 128, k = 10         4.11 -> 2.1 ms
-//   K3, FP8 band  100K x 50K,              d = 128, k = 10         4.77 -> 1.15 ms
-//   K3, off grid  480K x 17.8K,            d = 200, k = 10         32.0 -> 1.65 ms
-//   K3, off grid  130K x 30K,              d = 100, k = 50, lists  11.0 -> 1.40 ms
+//   K3, grid      500K users x 100K items, d = 64,  k = 25         1.87 -> 0.76 ms
+//   K3, grid      2M x 500K,               d = 128, k = 10         4.11 -> 2.4 ms
+//   K3, FP8 band  100K x 50K,              d = 128, k = 10         4.77 -> 0.90 ms
+//   K3, off grid  480K x 17.8K,            d = 200, k = 10         32.0 -> 1.58 ms
+//   K3, off grid  130K x 30K,              d = 100, k = 50, lists  11.0 -> 1.29 ms
 //   K6, off grid  2.2M pairs, d = 200: 2.39 -> 0.93 ms;  grid, 8.1M pairs, d = 128: 2.1 -> 1.1 ms
 #include <cuda_runtime.h>
 
