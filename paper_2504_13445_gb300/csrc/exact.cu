@@ -136,10 +136,11 @@ __device__ __forceinline__ void fma4(float4& s, const float4& a, const float4& b
 // FMAs (d <= 256 over eight lanes of four columns), joined by two additions and three folds, so
 // the error is at most gamma_13 sum|u p| <= gamma_13 ||u|| ||p|| (Higham, "Accuracy and Stability
 // of Numerical Algorithms", Section 3.1); 2^-20 = 16 * 2^-24 also covers the rounding of the FP64
-// reference sum, and 2^-140 underflow.  The item norm is bounded by the first item tile's
-// largest, widened by the width 2^-7 of a norm bucket (the order inside a bucket is free).
+// reference sum, and 2^-140 underflow.  Item norms are bounded by the end of the bucket of the first
+// item tile's largest: the order inside a bucket is free, and subnormal norms share buckets that are
+// wide for their size (all below 2^-133 one), so no factor of that largest norm would do.
 __device__ __forceinline__ float f32_bound(const ExactData& x, int64_t u) {
-    const float pn = __fmul_ru(*x.pmax, 1.0078125f);
+    const float pn = bucket_end(*x.pmax);
     return __fmaf_ru(__fmul_ru(x.unrm[u], 0x1p-20f), pn, 0x1p-140f);
 }
 

@@ -126,3 +126,27 @@ def test_users_per_warp(rkm, n):
             tau, tid, _ = ctx.thresholds(dev(U, -1), dev(W.P, -1), 5)
             np.testing.assert_array_equal(tid.cpu().numpy(), tid_o)
             np.testing.assert_allclose(tau.cpu().numpy(), tau_o, rtol=1e-12, atol=1e-300)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp8", "fp32"])
+def test_later_tiles_of_far_larger_subnormal_norms(rkm, prec):
+    """All norms below 2^-133 share one bucket, so the first item tile can hold norms of 2^-149 only
+    and a later one 32,764 times that.  The FP32 error bound must cover the later ones: the scores
+    of a user lie so close that FP32 sums put them in another order than FP64 ones."""
+    rng = np.random.default_rng(8)
+    unit = np.float32(2.0 ** -149)
+    P = np.zeros((2900, 64), np.float32)
+    P[np.arange(2500), rng.integers(0, 64, 2500)] = unit
+    codes = np.full((400, 64), 4095.0)
+    for row in codes:
+        row[rng.permutation(64)[:32]] += 1.0
+    P[2500:] = (codes * 2.0 ** -149).astype(np.float32)
+    # Entries 2^49 (1 + r 2^-19), r < 2^17: off the grid, sums exact in FP64.
+    U = ((2.0 ** 19 + rng.integers(0, 1 << 17, size=(150, 64))) * 2.0 ** 30).astype(np.float32)
+    with rkm.Context(prec) as ctx:
+        for k in (1, 20):
+            check(ctx, U, P, k)
+            assert ctx.stats()["exact_integer_path"] == 0
+            tau_o, _, _ = oracle.kmips(U, P, k)
+            np.testing.assert_array_equal(ctx.query_new_items(dev(P, -1)).cpu().numpy(),
+                                          oracle.query_new_items(U, tau_o, P))
