@@ -31,6 +31,7 @@
 #include "kernels.h"
 #include "state_io.h"
 #include "tmap.h"
+#include "unit_rule.h"
 
 using rkm::TmapPair;
 using rkm::make_tmaps;
@@ -152,9 +153,9 @@ struct rkm_ctx {
     cudaStream_t side[SIDES] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[SIDES] = {};
     size_t total_mem = 0;  // device memory, bytes
-    // Tunables (set by the autotuner for batches): user tiles per counting work unit, and the
-    // minimum number of items in the first counting stage of the filtered top-N.
-    int count_group = 32;
+    // Tunables (set by the autotuner for batches): the rule of user tiles per counting work unit, and
+    // the minimum number of items in the first counting stage of the filtered top-N.
+    rkm::UnitRule units;
     int64_t stage1_items = 8192;
     int64_t band_cap = 0;
     // phase timing (opts.profile)
@@ -815,15 +816,6 @@ rkm_status count_descriptor(const PathShape& ps, int64_t n, const UserOrder& uo,
     return RKM_OK;
 }
 
-// User tiles per counting work unit: the context's (32, or the autotuner's), or fewer where that
-// would leave the SMs less than about 8 units each.  2,000 users x 1,000 items made 4 units of 16
-// tiles (counting phase 78 us on 4 SMs; 64 units of one tile: 17 us), and 32 candidates against a
-// million users 244 units for 152 SMs.  Smaller units than needed reload the resident item tile more often.
-int unit_tiles(const rkm_ctx* c, int64_t n, int item_tiles) {
-    const int64_t tiles = (n + BU - 1) / BU * item_tiles;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(c->count_group, tiles / ((int64_t)c->num_sms * 8)));
-}
-
 // One counting stage over item tiles [t_begin, t_end) (t_end from the device if t_end_dev).
 rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrder& uo, const ItemSide& it,
                        bool new_items, int t_begin, int t_end, bool t_end_from_dev, const ExactData& x,
@@ -832,7 +824,7 @@ rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrd
     unsigned* unit_off;
     TRY(c->ensure(c->nprefix, std::max<int64_t>(it.tiles, 1), &nprefix));
     TRY(c->ensure(c->unit_off, it.tiles + 2, &unit_off));
-    const int group = unit_tiles(c, n, (t_end_from_dev ? (int)it.tiles : t_end) - t_begin);
+    const int group = c->units.tiles((n + BU - 1) / BU, (t_end_from_dev ? (int)it.tiles : t_end) - t_begin, c->num_sms);
     Phase ph_count(c, s, RKM_PHASE_COUNT);
     launch_build_units(it.tmax, uo.ucum, t_begin, t_end, t_end_from_dev ? &c->st->t_end : nullptr, BU, group,
                        nprefix, unit_off, (unsigned)c->band_cap, c->st, s);
@@ -1720,7 +1712,7 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
         j.tiles = tiles;
         j.t0 = c->opts.filter ? (int)std::min<int64_t>(tiles, (c0 + x.ps.item_tile - 1) / x.ps.item_tile) : tiles;
         j.tile_items = x.ps.item_tile;
-        j.group = sc->count_group;
+        j.group = sc->units.most;  // fixed: batch_units
         j.counts = x.cp.cnt;
         j.band = band;
         j.band_cap = (unsigned)sc->band_cap;
@@ -1944,12 +1936,13 @@ rkm_status tune_instance(rkm_ctx* sc, const rkm_instance& I, cudaStream_t s, Tun
         }
         return RKM_OK;
     };
+    const bool tc = path_shape(sc->opts.precision, I.d).tc;
     float best_ms = 1e30f;
     *best = TuneChoice{32, 8192};
     rkm_status r = RKM_OK;
     for (int g : groups) {
         for (int64_t st1 : stages) {
-            sc->count_group = g;
+            sc->units = batch_units(g, tc);
             sc->stage1_items = st1;
             float ms = 0.f;
             if ((r = run(&ms)) != RKM_OK) break;
@@ -2007,8 +2000,8 @@ extern "C" rkm_status rkm_topn_batch(rkm_ctx* c, const rkm_instance* inst, int c
         }
         const int g = (f != c->tune.end()) ? f->second.group : 32;
         const int64_t s1 = (f != c->tune.end()) ? f->second.stage1 : 8192;
-        if (sc->count_group != g || sc->stage1_items != s1) drop_graph(c);
-        sc->count_group = g;
+        if (sc->units.most != g || sc->stage1_items != s1) drop_graph(c);
+        sc->units = batch_units(g, path_shape(c->opts.precision, inst[i].d).tc);
         sc->stage1_items = s1;
     }
     if (tuned_any) save_tune_table(c);
