@@ -150,3 +150,22 @@ def test_later_tiles_of_far_larger_subnormal_norms(rkm, prec):
             tau_o, _, _ = oracle.kmips(U, P, k)
             np.testing.assert_array_equal(ctx.query_new_items(dev(P, -1)).cpu().numpy(),
                                           oracle.query_new_items(U, tau_o, P))
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 60])
+@pytest.mark.parametrize("k", [1, 25])
+def test_norms_and_sums_beyond_fp32(rkm, scale, k):
+    """Users off the grid whose squared norms overflow FP32: no FP32 bound holds, so FP64 ranks all
+    candidates and decides all pairs.  With items of 2^60 the FP32 sums overflow as well.  Entries are
+    positive, so that the products overflow to infinity and not to NaN."""
+    rng = np.random.default_rng(9)
+    U, P = np.abs(fine(rng, 130, 40)) * np.float32(2.0 ** 70), np.abs(fine(rng, 400, 40)) * np.float32(scale)
+    P[200:210] = P[190:200]  # equal scores: ids decide
+    with rkm.Context("bf16") as ctx:
+        check(ctx, U.astype(np.float32), P.astype(np.float32), k)
+        assert ctx.stats()["exact_integer_path"] == 0
+        tau_o, _, topk_o = oracle.kmips(U, P, k)
+        ids, top = ctx.topn(dev(U, -1), dev(P, -1), k, 50)[:2]
+        ids_o, top_o = oracle.topn(oracle.scores_histogram(topk_o, 400), 50)
+        np.testing.assert_array_equal(ids.cpu().numpy(), ids_o)
+        np.testing.assert_array_equal(top.cpu().numpy(), top_o)

@@ -39,3 +39,18 @@ def test_parts(rkm, n, m, d, k):
         ids, sc = ctx.topn(Ud, Pd, k, min(m, 20))[:2]
         np.testing.assert_array_equal(sc.cpu().numpy(), np.sort(want)[::-1][:min(m, 20)])
         np.testing.assert_array_equal(want[ids.cpu().numpy()], sc.cpu().numpy())
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("n,m,d,k,N", [(129, 300, 3, 10, 300), (500, 1_025, 8, 25, 400), (2_001, 3_000, 9, 5, 1_500)])
+def test_top_n_ids_among_equal_scores(rkm, prec, n, m, d, k, N):
+    """Most items share their score with others, and N cuts through such a group: ids decide."""
+    rng = np.random.default_rng(n)
+    U = rng.integers(-9, 10, size=(n, d)).astype(np.float32)
+    P = rng.integers(-9, 10, size=(m, d)).astype(np.float32)
+    _, _, topk_o = oracle.kmips(U, P, k)
+    ids_o, top_o = oracle.topn(oracle.scores_histogram(topk_o, m), N)
+    with rkm.Context(prec) as ctx:
+        ids, top = ctx.topn(torch.from_numpy(U).cuda(), torch.from_numpy(P).cuda(), k, N)[:2]
+    np.testing.assert_array_equal(ids.cpu().numpy(), ids_o)
+    np.testing.assert_array_equal(top.cpu().numpy(), top_o)
