@@ -522,7 +522,7 @@ rkm_status prep_items(rkm_ctx* c, const PathShape& ps, const float* P, int64_t m
     TRY(c->ensure(c->hist, HIST_WORDS, &hist));
     TRY(c->ensure(c->offs, NBUCKET, &offs));
     TRY(c->ensure(bb.perm, m, &it->perm));
-    launch_bucket_sort(it->rp.nrm, m, true, hist, offs, it->perm, nullptr, s);
+    launch_bucket_sort(it->rp.nrm, m, true, hist, offs, it->perm, nullptr, c->num_sms, s);
     const int64_t nt = std::max<int64_t>(it->tiles, 1);
     it->texp = nullptr;
     if (ps.fp8) {
@@ -651,7 +651,7 @@ void threshold_exact(rkm_ctx* c, const float* U, int64_t ldu, const float* P, in
     ExactData x{U, ldu, up.e, up.q, P, ldp, it.rp.e, it.rp.q, d, (int)round_up(d, 8), &c->st->off_grid,
                 pl.a.n, it.m, up.nrm, it.tmax};
     launch_exact_tau(x, pl.cand, pl.cand_cnt, pl.lfin, pl.cap, pl.nseg, it.perm, pl.a.n, pl.a.k, tau, tid, topk,
-                     c->st, s, pl.a.uperm);
+                     c->st, c->num_sms, s, pl.a.uperm);
 }
 
 // Seed order of the tensor-core threshold pass.  Items arrive in descending norm order and a
@@ -696,7 +696,7 @@ rkm_status threshold_seed_order(rkm_ctx* c, const PathShape& ps, const float* U,
     {
         Phase ph(c, s, RKM_PHASE_PREP);
         launch_seed_ratio(seed, up.nrm, n, r, s);
-        launch_bucket_sort(r, n, false, hist, offs, perm, nullptr, s);
+        launch_bucket_sort(r, n, false, hist, offs, perm, nullptr, c->num_sms, s);
         TRY(pack(c, ps, U, n, ldu, d, perm, pl->n_pad, c->u_pack, &pl->apack, s, up.e));
     }
     pl->a.A = pl->apack;
@@ -794,7 +794,7 @@ rkm_status order_users(rkm_ctx* c, const PathShape& ps, const float* U, int64_t 
     TRY(c->ensure(bb.perm, n, &uo->uperm));
     TRY(c->ensure(bb.cum, NBUCKET, &uo->ucum));
     launch_user_ratio(tau, up.n2, n, r, s);
-    launch_bucket_sort(r, n, false, hist, offs, uo->uperm, uo->ucum, s);
+    launch_bucket_sort(r, n, false, hist, offs, uo->uperm, uo->ucum, c->num_sms, s);
     const int64_t n_pad = round_up(std::max<int64_t>(n, 1), BU);
     TRY(pack(c, ps, U, n, ldu, d, uo->uperm, n_pad, bb.pack, &uo->pack, s, up.e));
     TRY(c->ensure(bb.meta, n, &uo->meta));
@@ -867,7 +867,8 @@ rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrd
 rkm_status band_stage(rkm_ctx* c, const ItemSide& it, bool new_items, const ExactData& x, const double* tau,
                       const int* tid, int* cnt, int2* band, cudaStream_t s) {
     Phase ph(c, s, RKM_PHASE_BAND);
-    launch_band_rescore(x, band, (unsigned)c->band_cap, it.perm, it.m, tau, tid, new_items, cnt, c->st, s);
+    launch_band_rescore(x, band, (unsigned)c->band_cap, it.perm, it.m, tau, tid, new_items, cnt, c->st, c->num_sms,
+                        s);
     return RKM_OK;
 }
 
@@ -1387,7 +1388,7 @@ rkm_status rkm_item_bounds(rkm_ctx* c, const float* U, int64_t n, int64_t ldu, c
     TRY(c->ensure(c->uperm, std::max<int64_t>(n, 1), &uperm));
     TRY(c->ensure(c->ucum, NBUCKET, &ucum));
     launch_user_ratio(tau, up.n2, n, r, s);
-    launch_bucket_sort(r, n, false, hist, offs, uperm, ucum, s);
+    launch_bucket_sort(r, n, false, hist, offs, uperm, ucum, c->num_sms, s);
     launch_item_uscore(pp.nrm, m, ucum, uscore, s);
     TRY(read_status(c, s));
     return RKM_OK;
@@ -1689,7 +1690,7 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
     // The exact thresholds read only the fields set so far; the later copy of the completed
     // jobs only adds fields, so either copy may read the staging at any time.
     CUDA_TRY(cudaMemcpyAsync(jd, J, (size_t)count * sizeof(BatchJob), cudaMemcpyHostToDevice, s));
-    launch_exact_tau_multi(jd, count, users, s);
+    launch_exact_tau_multi(jd, count, users, c->num_sms, s);
     const bool fp8 = w[0].ps.fp8;
     TRY(fork_sides(c, s));
     const auto prepare = [&](int i) -> rkm_status {

@@ -960,9 +960,9 @@ void launch_histogram_prefix(const int* lists, int64_t n, int kmax, int k, int64
 
 // Users per warp of K3: 32 fill the lanes of the FP64 sums; fewer when that would leave less
 // than about two rounds of the 32 warps that an SM holds.
-static int users_per_warp(int64_t n) {
+static int users_per_warp(int64_t n, int num_sms) {
     int per = 32;
-    while (per > 1 && n < (int64_t)per * 152 * 64) per >>= 1;
+    while (per > 1 && n < (int64_t)per * num_sms * 64) per >>= 1;
     return per;
 }
 
@@ -973,9 +973,9 @@ static int exact_blocks(int64_t n, int per) {
 
 void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt, const unsigned* lfin_key,
                       int cap, int nseg, const int* item_perm, int64_t n, int k, double* tau, int* tid, int* topk,
-                      DevStatus* st, cudaStream_t s, const int* uperm) {
+                      DevStatus* st, int num_sms, cudaStream_t s, const int* uperm) {
     if (n <= 0) return;
-    const int per = users_per_warp(n);
+    const int per = users_per_warp(n, num_sms);
     note_launch();
     k_exact_tau<<<exact_blocks(n, per), 32 * EX_WARPS, 0, s>>>(
         x, CandLists{cand, cand_cnt, lfin_key, cap, nseg, item_perm}, n, k, per, tau, tid, topk, st, uperm);
@@ -983,15 +983,15 @@ void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt,
 
 void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap, const int* item_perm,
                          int64_t m_ids, const double* tau, const int* tid, bool new_items, int* counts,
-                         DevStatus* st, cudaStream_t s) {
+                         DevStatus* st, int num_sms, cudaStream_t s) {
     (void)m_ids;
     note_launch();
-    k_band_rescore<<<1216, 32 * BAND_WARPS, 0, s>>>(x, band, band_cap, item_perm, tau, tid, new_items, counts, st);
+    k_band_rescore<<<8 * num_sms, 32 * BAND_WARPS, 0, s>>>(x, band, band_cap, item_perm, tau, tid, new_items, counts, st);
 }
 
-void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users, cudaStream_t s) {
+void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users, int num_sms, cudaStream_t s) {
     if (total_users <= 0) return;
-    const int per = users_per_warp(total_users);
+    const int per = users_per_warp(total_users, num_sms);
     note_launch();
     k_exact_tau_multi<<<exact_blocks(total_users, per), 32 * EX_WARPS, 0, s>>>(jobs, count, total_users, per);
 }

@@ -59,7 +59,7 @@ void launch_pack_bf16(const float* X, int64_t rows, int64_t ld, int d, const int
 // when `descending`).  Writes perm[pos] = source index and, if cum != null, the
 // inclusive prefix count of each bucket (in sort order).  hist: HIST_WORDS uints scratch.
 void launch_bucket_sort(const float* keys, int64_t count, bool descending, unsigned* hist,
-                        unsigned* offs, int* perm, unsigned* cum, cudaStream_t s);
+                        unsigned* offs, int* perm, unsigned* cum, int num_sms, cudaStream_t s);
 
 // gathered[i] = src[perm[i]] for float / double / int arrays.
 void launch_gather_f32(const float* src, const int* perm, int64_t count, float* dst, cudaStream_t s);
@@ -187,13 +187,13 @@ struct ExactData {
 // lists are by threshold-pass row and uperm[row] is the original user (rows, outputs).
 void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt, const unsigned* lfin_key,
                       int cap, int nseg, const int* item_perm, int64_t n, int k,
-                      double* tau, int* tid, int* topk, DevStatus* st, cudaStream_t s,
+                      double* tau, int* tid, int* topk, DevStatus* st, int num_sms, cudaStream_t s,
                       const int* uperm = nullptr);
 
 // K6: rescore queued band pairs (orig user, sorted item pos) and add members to counts.
 void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap,
                          const int* item_perm, int64_t m_ids, const double* tau, const int* tid,
-                         bool new_items, int* counts, DevStatus* st, cudaStream_t s);
+                         bool new_items, int* counts, DevStatus* st, int num_sms, cudaStream_t s);
 
 // K8: scores by histogram of S_k(u) (the first Section 2.2 baseline).
 void launch_histogram(const int* topk, int64_t nk, int* scores, cudaStream_t s);
@@ -286,7 +286,7 @@ struct BatchJob {
     DevStatus* st;
 };
 // jobs: device array of `count` problems, user_begin = exclusive prefix of n (total_users).
-void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users, cudaStream_t s);
+void launch_exact_tau_multi(const BatchJob* jobs, int count, int64_t total_users, int num_sms, cudaStream_t s);
 // Zero every problem's counts and band counters (max_m: largest m).
 void launch_batch_reset(const BatchJob* jobs, int count, int64_t max_m, cudaStream_t s);
 // Unit lists of counting stage 1 (tiles [0, t0)) or 2 (tiles [t0, st->t_end)) of every problem.

@@ -585,7 +585,7 @@ void launch_pack_bf16(const float* X, int64_t rows, int64_t ld, int d, const int
 }
 
 void launch_bucket_sort(const float* keys, int64_t count, bool descending, unsigned* hist,
-                        unsigned* offs, int* perm, unsigned* cum, cudaStream_t s) {
+                        unsigned* offs, int* perm, unsigned* cum, int num_sms, cudaStream_t s) {
     constexpr int WORDS = SORT_WORDS * sizeof(unsigned), TABLE = SORT_CHUNK * sizeof(unsigned);
     if (count > 0 && count <= SORT_SMALL) {
         cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, WORDS);
@@ -595,7 +595,7 @@ void launch_bucket_sort(const float* keys, int64_t count, bool descending, unsig
     }
     // Keys per block: every SM busy, as far as a block's fixed work (clearing and scanning its
     // counters) stays below that on its keys.
-    const int chunk = (int)std::min<int64_t>(SORT_CHUNK, std::max<int64_t>(1024, (count + 147) / 148));
+    const int chunk = (int)std::min<int64_t>(SORT_CHUNK, std::max<int64_t>(1024, (count + num_sms - 1) / num_sms));
     cudaMemsetAsync(hist, 0, NBUCKET * sizeof(unsigned), s);
     if (count > 0) {
         cudaFuncSetAttribute(k_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, WORDS);
