@@ -818,8 +818,7 @@ rkm_status count_descriptor(const PathShape& ps, int64_t n, const UserOrder& uo,
 
 // One counting stage over item tiles [t_begin, t_end) (t_end from the device if t_end_dev).
 rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrder& uo, const ItemSide& it,
-                       bool new_items, int t_begin, int t_end, bool t_end_from_dev, const ExactData& x,
-                       const double* tau, const int* tid, int* cnt, int2* band, cudaStream_t s) {
+                       int t_begin, int t_end, bool t_end_from_dev, int* cnt, int2* band, cudaStream_t s) {
     int* nprefix;
     unsigned* unit_off;
     TRY(c->ensure(c->nprefix, std::max<int64_t>(it.tiles, 1), &nprefix));
@@ -835,9 +834,6 @@ rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrd
     a.m = it.m;
     a.dp = ps.dp;
     a.meta = uo.meta;
-    a.item_id = new_items ? nullptr : it.perm;
-    a.new_items = new_items;
-    a.tmax = it.tmax;
     a.thmax = it.thmax;
     a.tdel = it.tdel;
     a.texp = it.texp;
@@ -867,8 +863,7 @@ rkm_status count_stage(rkm_ctx* c, const PathShape& ps, int64_t n, const UserOrd
 rkm_status band_stage(rkm_ctx* c, const ItemSide& it, bool new_items, const ExactData& x, const double* tau,
                       const int* tid, int* cnt, int2* band, cudaStream_t s) {
     Phase ph(c, s, RKM_PHASE_BAND);
-    launch_band_rescore(x, band, (unsigned)c->band_cap, it.perm, it.m, tau, tid, new_items, cnt, c->st, c->num_sms,
-                        s);
+    launch_band_rescore(x, band, (unsigned)c->band_cap, it.perm, tau, tid, new_items, cnt, c->st, c->num_sms, s);
     return RKM_OK;
 }
 
@@ -961,7 +956,7 @@ rkm_status rkm::query_resident(rkm_ctx* c, const rkm_ctx* r, const float* Q, int
         CUDA_TRY(cudaMemsetAsync(&c->st->band_count, 0, 2 * sizeof(unsigned), s));
         const double* rtau = static_cast<const double*>(r->res_tau.p);
         const int* rtid = static_cast<const int*>(r->res_tid.p);
-        TRY(count_stage(c, ps, n, uo, it, true, 0, (int)it.tiles, false, x, rtau, rtid, cnt, band, s));
+        TRY(count_stage(c, ps, n, uo, it, 0, (int)it.tiles, false, cnt, band, s));
         TRY(band_stage(c, it, true, x, rtau, rtid, cnt, band, s));
         scatter_i32(cnt, it.perm, q, counts, s);
         TRY(read_status(c, s));
@@ -1125,7 +1120,7 @@ rkm_status count_enqueue(rkm_ctx* c, const PathShape& ps, int64_t n, const ItemS
     CUDA_TRY(cudaMemsetAsync(&c->st->band_count, 0, 2 * sizeof(unsigned), s));  // band_count, band_done
     const int tiles = (int)it.tiles;
     if (!filter) {
-        TRY(count_stage(c, ps, n, uo, it, false, 0, tiles, false, x, tau, tid, cnt, band, s));
+        TRY(count_stage(c, ps, n, uo, it, 0, tiles, false, cnt, band, s));
         TRY(band_stage(c, it, false, x, tau, tid, cnt, band, s));
         Phase ph(c, s, RKM_PHASE_TOPN);
         if (scores) scatter_i32(cnt, it.perm, it.m, scores, s);
@@ -1136,7 +1131,7 @@ rkm_status count_enqueue(rkm_ctx* c, const PathShape& ps, int64_t n, const ItemS
     // and a few thousand more; its N-th score is an exact lower bound of the final one.
     const int64_t c0 = std::max<int64_t>(4 * (int64_t)N, c->stage1_items);
     const int t0 = (int)std::min<int64_t>(tiles, (c0 + ps.item_tile - 1) / ps.item_tile);
-    TRY(count_stage(c, ps, n, uo, it, false, 0, t0, false, x, tau, tid, cnt, band, s));
+    TRY(count_stage(c, ps, n, uo, it, 0, t0, false, cnt, band, s));
     TRY(band_stage(c, it, false, x, tau, tid, cnt, band, s));
     int *tids_c0, *tsc_c0;
     TRY(c->ensure(c->top_ids, N, &tids_c0));
@@ -1148,7 +1143,7 @@ rkm_status count_enqueue(rkm_ctx* c, const PathShape& ps, int64_t n, const ItemS
             launch_topn(cnt, it.perm, m0, nullptr, N, tids_c0, tsc_c0, c->st, s);
             launch_filter_cut(tsc_c0, N, it.tmax, uo.ucum, it.tiles, t0, ps.item_tile, it.m, c->st, s);
         }
-        TRY(count_stage(c, ps, n, uo, it, false, t0, 0, true, x, tau, tid, cnt, band, s));
+        TRY(count_stage(c, ps, n, uo, it, t0, 0, true, cnt, band, s));
         TRY(band_stage(c, it, false, x, tau, tid, cnt, band, s));
         Phase ph(c, s, RKM_PHASE_TOPN);
         launch_topn(cnt, it.perm, it.m, &c->st->m_counted, N, ids, top_scores, c->st, s);
@@ -1726,9 +1721,6 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
         a.m = x.it.m;
         a.dp = x.ps.dp;
         a.meta = x.cp.uo.meta;
-        a.item_id = x.it.perm;
-        a.new_items = false;
-        a.tmax = x.it.tmax;
         a.thmax = x.it.thmax;
         a.tdel = x.it.tdel;
         a.texp = x.it.texp;

@@ -539,7 +539,7 @@ __device__ __forceinline__ int collect(const ExactData& x, const CandLists& l, E
 // upper bound reaches it are scored at all (546 candidates per user became 99 at 100K x 50K,
 // d = 128, k = 10, FP8).
 __device__ __forceinline__ int best_of_many(const ExactData& x, bool grid, const CandLists& l, ExactWarp& S, int k,
-                                         DevStatus* st, int64_t u, int64_t uo, bool vec, int lane, float L, int eu,
+                                         DevStatus* st, int64_t u, bool vec, int lane, float L, int eu,
                                          float err) {
     bool bad = !(err < INFINITY);
     unsigned scored = 0;
@@ -618,7 +618,7 @@ __device__ __forceinline__ int exact_user(const ExactData& x, bool grid, const C
     int seg = 0, base = 0;
     int n = collect(x, l, S, u, L, INFINITY, 0, EX_CHUNK - 32, seg, base, lane, st);
     if (seg < l.nseg) {
-        n = best_of_many(x, grid, l, S, k, st, u, uo, vec, lane, L, eu, err);
+        n = best_of_many(x, grid, l, S, k, st, u, vec, lane, L, eu, err);
         scored += S.more;
         bad = S.bad != 0;
         keyed = grid;
@@ -982,9 +982,8 @@ void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt,
 }
 
 void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap, const int* item_perm,
-                         int64_t m_ids, const double* tau, const int* tid, bool new_items, int* counts,
+                         const double* tau, const int* tid, bool new_items, int* counts,
                          DevStatus* st, int num_sms, cudaStream_t s) {
-    (void)m_ids;
     note_launch();
     k_band_rescore<<<8 * num_sms, 32 * BAND_WARPS, 0, s>>>(x, band, band_cap, item_perm, tau, tid, new_items, counts, st);
 }

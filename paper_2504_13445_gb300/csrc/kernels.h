@@ -61,11 +61,6 @@ void launch_pack_bf16(const float* X, int64_t rows, int64_t ld, int d, const int
 void launch_bucket_sort(const float* keys, int64_t count, bool descending, unsigned* hist,
                         unsigned* offs, int* perm, unsigned* cum, int num_sms, cudaStream_t s);
 
-// gathered[i] = src[perm[i]] for float / double / int arrays.
-void launch_gather_f32(const float* src, const int* perm, int64_t count, float* dst, cudaStream_t s);
-void launch_gather_f64(const double* src, const int* perm, int64_t count, double* dst, cudaStream_t s);
-void launch_gather_i32(const int* src, const int* perm, int64_t count, int* dst, cudaStream_t s);
-
 // Per tile t of sorted positions [t*tile, min(count,(t+1)*tile)): the maxima of nrm, nhat and
 // del over the rows perm[pos] (0 for an empty tile).
 void launch_tile_max(const float* nrm, const float* nhat, const float* del, const int* perm, int64_t count,
@@ -192,7 +187,7 @@ void launch_exact_tau(const ExactData& x, const Cand* cand, const int* cand_cnt,
 
 // K6: rescore queued band pairs (orig user, sorted item pos) and add members to counts.
 void launch_band_rescore(const ExactData& x, const int2* band, unsigned band_cap,
-                         const int* item_perm, int64_t m_ids, const double* tau, const int* tid,
+                         const int* item_perm, const double* tau, const int* tid,
                          bool new_items, int* counts, DevStatus* st, int num_sms, cudaStream_t s);
 
 // K8: scores by histogram of S_k(u) (the first Section 2.2 baseline).
@@ -209,9 +204,6 @@ struct CountArgs {
     int64_t n, m;
     int dp;
     const UserMeta* meta;   // [n] per-user record, ratio order
-    const int* item_id;     // sorted pos -> original item id (null for new items)
-    bool new_items;         // strict rule u.p > tau_u (new ids beat no tie)
-    const float* tmax;      // per item tile: max ||p||
     const float* thmax;     // per item tile: max ||p^||
     const float* tdel;      // per item tile: max ||p^ - p||
     const int* texp;        // per item tile: FP8 tile exponent (unused for BF16 / FP32)

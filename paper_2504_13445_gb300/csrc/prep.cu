@@ -449,14 +449,6 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fix(const unsigned* __restr
     if (cum) cum[i] = o + hist[i];
 }
 
-template <typename T>
-__global__ void k_gather(const T* __restrict__ src, const int* __restrict__ perm, int64_t count,
-                         T* __restrict__ dst) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = src[perm[i]];
-}
-
 // Per tile of `tile` consecutive sorted rows: max ||p||, max ||p^||, max ||p^ - p||.
 __global__ void k_tile_max(const float* __restrict__ nrm, const float* __restrict__ nhat,
                            const float* __restrict__ del, const int* __restrict__ perm, int64_t count, int tile,
@@ -611,25 +603,6 @@ void launch_bucket_sort(const float* keys, int64_t count, bool descending, unsig
         note_launch();
         k_scatter<<<grid_for(count, chunk, 1024), SORT_THREADS, WORDS + TABLE, s>>>(keys, count, chunk, descending,
                                                                                     offs, perm);
-    }
-}
-
-void launch_gather_f32(const float* src, const int* perm, int64_t count, float* dst, cudaStream_t s) {
-    if (count > 0) {
-        note_launch();
-        k_gather<float><<<grid_for(count, 256, 65536), 256, 0, s>>>(src, perm, count, dst);
-    }
-}
-void launch_gather_f64(const double* src, const int* perm, int64_t count, double* dst, cudaStream_t s) {
-    if (count > 0) {
-        note_launch();
-        k_gather<double><<<grid_for(count, 256, 65536), 256, 0, s>>>(src, perm, count, dst);
-    }
-}
-void launch_gather_i32(const int* src, const int* perm, int64_t count, int* dst, cudaStream_t s) {
-    if (count > 0) {
-        note_launch();
-        k_gather<int><<<grid_for(count, 256, 65536), 256, 0, s>>>(src, perm, count, dst);
     }
 }
 

@@ -231,37 +231,9 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-// Issue a load of 32 consecutive FP32 columns of this thread's TMEM lane (warp-collective);
-// the registers are valid only after tmem_wait_bind on the same array.
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
-          "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
-          "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-
-// Wait for every outstanding tcgen05.ld of this thread; the "+r" operands make every later
-// use of r depend on the wait, so no use can be scheduled before the data has arrived.
-__device__ __forceinline__ void tmem_wait_bind(uint32_t (&r)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
-                   "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]),
-                   "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]),
-                   "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-                 :
-                 : "memory");
-}
-
-// tcgen05.ld with the .red qualifier of sm_103a: the same 32 columns as tmem_ld32_issue and,
-// in mx, their maximum along this thread's row, computed by the load itself (no reduction
-// tree in the epilogue).  r and mx are valid only after tmem_wait_bind_max on them.
+// Issue a load of 32 consecutive FP32 columns of this thread's TMEM lane (warp-collective) by
+// tcgen05.ld with the .red qualifier of sm_103a: mx gets their maximum, computed by the load
+// itself (no reduction tree in the epilogue).  r and mx are valid only after tmem_wait_bind_max.
 __device__ __forceinline__ void tmem_ld32_max_issue(uint32_t taddr, uint32_t (&r)[32], float& mx) {
     asm volatile(
         "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
@@ -276,7 +248,8 @@ __device__ __forceinline__ void tmem_ld32_max_issue(uint32_t taddr, uint32_t (&r
         : "memory");
 }
 
-// Wait for every outstanding tcgen05.ld of this thread, binding r and mx as tmem_wait_bind does.
+// Wait for every outstanding tcgen05.ld of this thread; the "+r" operands make every later use of r
+// and mx depend on the wait, so no use can be scheduled before the data has arrived.
 __device__ __forceinline__ void tmem_wait_bind_max(uint32_t (&r)[32], float& mx) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
