@@ -101,16 +101,19 @@ typedef struct {
                                 accumulator tile back (0 = auto, 2, or 4: four split every
                                 tile's columns between two groups, doubling the reads in
                                 flight).  Auto: 2 for the threshold pass; for the counting
-                                pass 4 when a tile is one K-block deep (BF16 d <= 64, FP8
-                                d <= 128), else 2.  The threshold pass takes 4 only when
-                                asked and four per-user heaps of k bounds fit (k <= 32).   */
+                                pass 4 for BF16 tiles one K-block deep (d <= 64), else 2 (a
+                                batch's counting launch: always 2).  The threshold pass takes
+                                4 only when asked and four per-user heaps of k bounds fit
+                                (k <= 32).                                                 */
     int seed_order;          /* tensor-core threshold pass: 1 = first a pass over the highest-norm
                                 items (512 to 4,096 of them) gives each user a lower bound of
                                 tau_u, users are grouped into tiles by bound / ||u|| and the bound
                                 seeds the selector, so each tile's Cauchy-Schwarz stop comes
                                 sooner and fewer candidates are recorded (default; used when the
-                                users fit one launch and the items are at least six times those
-                                of the seed pass); 0 = users in input order               */
+                                users fit one launch, the items are at least six times those of
+                                the seed pass and it has 2 k bounds to take the k-th of, one per
+                                16 items, 128 at most; batches take the bounds but keep their
+                                users in input order); 0 = users in input order           */
 } rkm_opts;
 
 /* Phases timed when rkm_opts.profile is set (indices of rkm_stats.phase_ms). */

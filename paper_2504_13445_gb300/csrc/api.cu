@@ -897,7 +897,8 @@ int64_t grown_band_cap(const rkm_ctx* c) {
 void init_caps(rkm_ctx* c, int64_t n, int k) {
     // FP8's guard band is about eight times BF16's, so its lists start larger: at 100K x 50K, k = 10,
     // some users need more than 352 slots (8 k + 256) per segment, and the overflow, a compaction
-    // per hit and a second pass made a context's first call 40 ms instead of 6.
+    // per hit and a second pass made a context's first call 40 ms instead of 6.  A rule in k alone: a
+    // larger catalogue can still overflow it once (500K x 100K, k = 25: 30 ms, then 22).
     const int dflt = c->opts.precision == RKM_FP8 ? 16 * k + 512 : 2 * k + 96;
     int cap = c->opts.cand_capacity > 0 ? c->opts.cand_capacity : (int)round_up(dflt, 32);
     cap = (int)round_up(cap, 32);

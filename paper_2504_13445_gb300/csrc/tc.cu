@@ -1219,19 +1219,22 @@ void launch_threshold_ng(const TcInstance* inst, int count, long long total_unit
 
 }  // namespace
 
-// Two groups unless four are asked for: measured on GB300 (BF16, d = 64 and 128), four
-// groups made the threshold pass 1.5-1.8x slower.  Each group's heap then sees a quarter of
-// the items, so its bound is lower and it records more candidates (exact rescoring took 2.4x
-// longer), and 18 warps leave 96 registers per thread, so the hit path spills.
+// Two groups unless four are asked for.  Threshold phase on GB300 with two / four groups, ms:
+//   500K x 100K, d = 64,  k = 25   4.33 / 8.85      200K x 50K, d = 32,  k = 10   0.67 / 0.84
+//   500K x 100K, d = 64,  k = 10   2.91 / 4.22      300K x 100K, d = 128, k = 10  3.33 / 6.24
+// All groups share seed and published bounds, so four record 1 to 8 % more candidates only; 18 warps
+// leave 96 registers per thread, and the hit path spills (206 bytes; none at 168 registers).
 int threshold_groups(int kheap, int max_dp, bool fp8, int want) {
     if (want != 4 || kheap > 32) return 2;
     return threshold_layout(4, kheap, max_dp, fp8, false).slots >= 2 ? 4 : 2;
 }
 
 // Four groups for BF16 tiles one K-block deep (d <= 64): the MMA of a tile is then shortest and
-// eight warps reading each tile made the counting pass 15 % faster at d = 64 on GB300; at two
-// K-blocks and more the two were equal.  FP8 keeps two: its descale multiplies make the
-// four-group kernel (96 registers per thread) spill, and it ran 2.7x slower.
+// eight warps reading each tile make the counting phase 10 to 13 % shorter on GB300 (500K x 100K,
+// d = 64: 3.20 -> 2.88 ms; 200K x 50K, d = 32: 0.43 -> 0.37); at two K-blocks the two are equal (300K x
+// 100K, d = 128: 2.93 and 2.94).  FP8 keeps two, by a figure from before hits became bit masks (2.7x
+// slower with four, by spills); with them four measure 0.76 -> 0.62 ms at 100K x 50K, d = 128, 4.49 ->
+// 3.81 at 500K x 100K, d = 64, and 2.14 -> 1.86 at 200K x 50K, d = 200.
 int count_groups(int dp, bool fp8, int want) {
     if (want == 2 || want == 4) return want;
     return (!fp8 && dp <= 64) ? 4 : 2;
