@@ -1709,7 +1709,7 @@ rkm_status batch_enqueue_tc(rkm_ctx* c, const rkm_instance* inst, int count, std
         j.tiles = tiles;
         j.t0 = c->opts.filter ? (int)std::min<int64_t>(tiles, (c0 + x.ps.item_tile - 1) / x.ps.item_tile) : tiles;
         j.tile_items = x.ps.item_tile;
-        j.group = sc->units.most;  // fixed: batch_units
+        j.group = sc->units.tiles((I.n + BU - 1) / BU, tiles, c->num_sms);
         j.counts = x.cp.cnt;
         j.band = band;
         j.band_cap = (unsigned)sc->band_cap;

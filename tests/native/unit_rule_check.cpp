@@ -23,6 +23,8 @@ int main() {
                 // FP32 batches launch each instance by itself, under the single call's rule.
                 CHECK(rkm::batch_units(g, false).tiles(users, items, 152) == (rkm::UnitRule{g, false}).tiles(users, items, 152));
             }
+            // A stored choice is read from a text file: no value makes an empty unit.
+            for (int g : {0, -5}) CHECK(rkm::batch_units(g, true).tiles(users, items, 152) == 1);
             const int t = rkm::UnitRule{}.tiles(users, items, 152);
             CHECK(t >= 1 && t <= 32);
             CHECK(t == 1 || (long long)t * 152 * 8 <= users * items);
